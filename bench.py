@@ -86,6 +86,8 @@ STEP_KERNEL_SOURCES = [
     "paper_1908_10793_gb300/csrc/dust_step_kernels.cuh",
     "paper_1908_10793_gb300/csrc/dust_tiled.cuh",
     "paper_1908_10793_gb300/csrc/dust_slab.cuh",
+    "paper_1908_10793_gb300/csrc/dust_cube.cuh",
+    "paper_1908_10793_gb300/csrc/dust_cube_math.cuh",
     "paper_1908_10793_gb300/csrc/dust_geom_sb.cu",
 ]
 

@@ -878,7 +878,7 @@ cudaError_t launch_step_geom(const StepArgs<Real> &a, int weight, int kernel,
     ta.count_out = count_out;
     ta.perm = perm;
     ta.perm_id = perm_id;
-    ta.dst = dst;
+    ta.dst = perm ? dst : a.s;
     if (kernel == DUST_KERNEL_PER_GRAIN) {
         if (perm) return cudaErrorInvalidValue;  // only the slab kernel gathers
         if constexpr (GEOM == GEOM_CYL || GEOM == GEOM_SPH)

@@ -136,7 +136,7 @@ struct TiledArgs {
     int32_t *count_out;           // [nkeys + 2], zeroed before the step
     // optional: the sort's gather fused into the step.  The grain at sorted
     // position i is read from s at perm[i] and written, with id perm_id[i],
-    // to dst at i (null: read and write s in place)
+    // to dst at i (null: read and write s in place; dst is then s)
     const int32_t *perm;
     const int32_t *perm_id;
     StoreDev<Real> dst;

@@ -1,4 +1,5 @@
-// Slab-group step kernel (mixed precision).  One CTA per tile of zones, the
+// Slab-group step kernel of two-dimensional grids (mixed precision; three-
+// dimensional ones: dust_cube.cuh).  One CTA per tile of zones, the
 // tile's gas stencil staged in shared memory.  A warp takes an equal range of
 // the tile's sort keys (zones), whose grains are contiguous in the store, and
 // walks it in passes of up to kSlabCap grains.
@@ -42,7 +43,7 @@ constexpr int kRecFields = 13;  // 3 x 3 weights, 4 deposit channels
 
 template <int FLAT>
 struct SlabShape {
-    // FLAT: 0 = three gridded directions, 1 = y not gridded, 2 = z not gridded
+    // FLAT: 1 = y not gridded, 2 = z not gridded
     static constexpr int NB = FLAT == 1 ? 1 : 3;
     static constexpr int NC = FLAT == 2 ? 1 : 3;
     static constexpr int BC = NB == 3 ? 1 : 0;   // index of the host node in y
@@ -280,7 +281,8 @@ __device__ __noinline__ int32_t slab_predict_key(const GridDev &g, const PhysDev
 // Returns false when the wait for the gas box ran out (DUST_FLAG_TIMEOUT).
 template <int GEOM, int FLAT, int MODE, int TX = 0, int TY = 0, int TZ = 0, bool PRED = false>
 __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int tile, const int ntile,
-                                          unsigned char *smem_raw, const bool reuse)
+                                          unsigned char *smem_raw, const bool reuse, const int part = 0,
+                                          const int parts = 1)
 {
     using Sh = SlabShape<FLAT>;
     constexpr int NB = Sh::NB, NC = Sh::NC;
@@ -312,7 +314,8 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
         // grains removed before the last sort sit after every zone's segment:
         // they keep the removed-grain key and are moved as they are
         const int D0 = TA.key_off[g.nkeys], D1 = (int)A.s.n;
-        for (int gi = D0 + tile * blockDim.x + threadIdx.x; gi < D1; gi += ntile * blockDim.x) {
+        const int vb = tile * parts + part, nvb = ntile * parts;
+        for (int gi = D0 + vb * blockDim.x + threadIdx.x; gi < D1; gi += nvb * blockDim.x) {
             if (TA.emit_keys) TA.key_out[gi] = (int32_t)g.nkeys;
             if (TA.perm) {
                 const int src = TA.perm[gi];
@@ -326,11 +329,13 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                 if (S.param) O.param[gi] = S.param[src];
             }
         }
-        if (TA.emit_keys && tile == 0 && threadIdx.x == 0 && D1 > D0)
+        if (TA.emit_keys && vb == 0 && threadIdx.x == 0 && D1 > D0)
             atomicAdd(&TA.count_out[g.nkeys], (int32_t)(D1 - D0));
     }
     const int64_t kbase = (int64_t)tile * tvol;
-    if (TA.key_off[kbase + tvol] <= TA.key_off[kbase]) return true;
+    // this block's zones: a part of the tile's
+    const int zb0 = (int)(((int64_t)part * tvol) / parts), zb1 = (int)(((int64_t)(part + 1) * tvol) / parts);
+    if (TA.key_off[kbase + zb1] <= TA.key_off[kbase + zb0]) return true;
 
     int B[3], o[3], tc[3];
     tc[0] = tile % g.nt[0];
@@ -412,33 +417,10 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
     __syncthreads();
     if (!gas_box_finish<float>(g, A.gas, TA.gas_tmap, sgas, o, B, sbar, A.status, TA.wait_ns)) return false;
 
-    // The deposit box.  In a tile of at most 65535 grains each word of the box
-    // takes at most one piece per grain, so a piece v with |v| < 2^31 is
-    // added exactly as two 32-bit counters that need no carry: the sum of
-    // the pieces' low 16 bits (unsigned, below 2^32) and of v >> 16 (signed,
-    // below 2^31 in size); the word is 65536 * high + low.  Both adds return
-    // nothing, so no lane waits for the shared-memory round trip.  Larger
-    // pieces go to the global deposit directly.  A denser tile keeps the box
-    // as int64 words added as two 32-bit atomics with the carry.
-    unsigned *blo = reinterpret_cast<unsigned *>(sdep);
-    int *bhi = reinterpret_cast<int *>(blo + 4 * bvol);
-    // Measured: the split form pays in the 3-D tiles (27 nodes per zone); the
-    // 2-D tiles of the batched x-z boxes ran 9% slower with it than with the
-    // int64 words, so the 2-D copies keep those.
-    const bool split = FLAT == 0 && skoff[tvol] - skoff[0] <= 65535;
-    auto box_add_split = [&](int ch, int lin, int v) {
-        atomicAdd(&blo[ch * bvol + lin], (unsigned)v & 0xffffu);
-        atomicAdd(&bhi[ch * bvol + lin], v >> 16);
-    };
-    auto box_add = [&](int ch, int lin, long long v) {
-        if (!split) {
-            shared_add_i64(&sdep[ch * bvol + lin], v);
-        } else if (v >= -2147483647LL && v <= 2147483647LL) {
-            box_add_split(ch, lin, (int)v);
-        } else {
-            box_piece_to_global(g, A.dep, o[0], o[1], o[2], B[0], B[1], lin, ch, v);
-        }
-    };
+    // The deposit box: int64 words added as two 32-bit atomics with the carry
+    // (the carry-free counters of the three-dimensional kernel were 9% slower
+    // here, with 9 nodes per zone).
+    auto box_add = [&](int ch, int lin, long long v) { shared_add_i64(&sdep[ch * bvol + lin], v); };
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
@@ -449,14 +431,14 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
     float moved = 0.f;
     bool big = false;
 
-    // Each warp takes an equal range [zw0, zw1) of the tile's zones (keys)
+    // Each warp takes an equal range [zw0, zw1) of the block's zones (keys)
     // and walks its grains, contiguous in the store, in passes of at most
     // kSlabCap grains that end on chunk boundaries (a zone's end, or its
     // start plus a multiple of kSlabCap), so each zone's part of a pass is
     // one whole chunk of its run and is quantised in that pass: nothing is
     // carried between passes.  A pass spans as many zones as its grains
     // fill; its owner phase takes them ten at a time.
-    const int zw0 = (warp * tvol) / nwarps, zw1 = ((warp + 1) * tvol) / nwarps;
+    const int zw0 = zb0 + (warp * (zb1 - zb0)) / nwarps, zw1 = zb0 + ((warp + 1) * (zb1 - zb0)) / nwarps;
     const int Gend = skoff[zw1];
     float *rb = srec + warp * (kRecFields * kRecStride);
     unsigned short *zt = sztab + warp * kSlabCap;
@@ -1095,36 +1077,14 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                         }
                 };
                 if (own) {
-                    if (narrow && split) {
-                        // the common form: 32-bit roundings, carry-free adds, and
-                        // 32-bit sums of the pieces (their sizes add up to at most
-                        // the chunk's bound, below 2^31)
-                        int ps32[4] = {0, 0, 0, 0};
-#pragma unroll
-                        for (int b = 0; b < NB; ++b)
-#pragma unroll
-                            for (int c = 0; c < NC; ++c) {
-                                if (a == 1 && b == Sh::BC && c == Sh::CC) continue;  // host: remainder
-                                const int lin =
-                                    (ohx + a - 1) + B[0] * ((ohy + b - Sh::BC) + B[1] * (ohz + c - Sh::CC));
-#pragma unroll
-                                for (int ch = 0; ch < NCH; ++ch) {
-                                    const float v = (ch & 1) ? acc[b][c][ch >> 1].y : acc[b][c][ch >> 1].x;
-                                    const int piece = __float2int_rn(v);
-                                    box_add_split(ch, lin, piece);
-                                    ps32[ch] += piece;
-                                }
-                            }
-#pragma unroll
-                        for (int ch = 0; ch < 4; ++ch) ps[ch] = ps32[ch];
-                    } else if (FLAT != 0 && narrow) {
-                        // 2-D tiles: 32-bit roundings into the int64 words
+                    if (narrow) {
+                        // 32-bit roundings into the int64 words
                         quantise([](float v) { return (long long)__float2int_rn(v); },
                                  [&](int ch, int lin, long long v) {
                                      shared_add_i64_always(&sdep[ch * bvol + lin], v);
                                  });
                     } else {
-                        // wide chunk sums, or a tile too dense for the split box
+                        // wide chunk sums
                         quantise([&](float v) {
                             big |= !(fabsf(v) < 4.5e15f);
                             return rround(v);
@@ -1157,8 +1117,7 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
         const int64_t gz = i + (int64_t)g.n[0] * (j + (int64_t)g.n[1] * k);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const long long v = split ? (long long)bhi[c * bvol + lin] * 65536 + (long long)blo[c * bvol + lin]
-                                      : (long long)sdep[c * bvol + lin];
+            const long long v = (long long)sdep[c * bvol + lin];
             if (v != 0) atomicAdd(&A.dep[4 * gz + c], (unsigned long long)v);
         }
     }
@@ -1176,12 +1135,42 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
     return true;
 }
 
+// Blocks per tile: a grid of few tiles leaves most of the chip idle (or its last
+// wave nearly empty), so its tiles are cut into ranges of zones.  Every part
+// stages the tile's gas box and flushes its own deposit box; the integers do
+// not depend on the cut (64^2 box of 16 tiles: step 74 -> 34 us; 50x37x29 box of
+// 140 tiles: 100 -> 70 us).  The number of parts with the smallest rounds x (fixed
+// + work / parts) is taken, with 2 resident blocks on each of 152 SMs; fixed: us
+// of a block's staging and flush, per_grain / per_zone: us of a tile's work
+// beside a second resident block (measured inside the kernels).
+inline int tile_parts(int64_t ntiles, int64_t n, int tvol, double fixed, double per_grain, double per_zone)
+{
+    const double work = per_grain * (double)n / (double)ntiles + per_zone * tvol;
+    int best = 1;
+    double least = 0.0;
+    for (int p = 1; p <= 8 && p <= tvol; p *= 2) {
+        const double t = (double)((ntiles * p + 303) / 304) * (fixed + work / p);
+        if (p == 1 || t < 0.95 * least) {
+            best = p;
+            least = t;
+        }
+    }
+    return best;
+}
+
+}  // namespace dust
+
+#include "dust_cube.cuh"
+
+namespace dust {
+
 template <int GEOM, int FLAT, int MODE, int TX = 0, int TY = 0, int TZ = 0>
 __global__ void __launch_bounds__(kSlabThreads, 2)
-step_slab_kernel(const __grid_constant__ TiledArgs<float> TA)
+step_slab_kernel(const __grid_constant__ TiledArgs<float> TA, const int parts)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    slab_tile<GEOM, FLAT, MODE, TX, TY, TZ>(TA, blockIdx.x, gridDim.x, smem_raw, false);
+    slab_tile<GEOM, FLAT, MODE, TX, TY, TZ>(TA, blockIdx.x / parts, gridDim.x / parts, smem_raw, false,
+                                            blockIdx.x % parts, parts);
 }
 
 // Gas predictor on the slab layout (Sec. 3.1): one tile per block, the
@@ -1189,21 +1178,20 @@ step_slab_kernel(const __grid_constant__ TiledArgs<float> TA)
 // for the others.
 template <int GEOM, int FLAT, int TX = 0, int TY = 0, int TZ = 0>
 __global__ void __launch_bounds__(kSlabThreads, 2)
-predict_slab_kernel(const __grid_constant__ TiledArgs<float> TA)
+predict_slab_kernel(const __grid_constant__ TiledArgs<float> TA, const int parts)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    slab_tile<GEOM, FLAT, 1, TX, TY, TZ, true>(TA, blockIdx.x, gridDim.x, smem_raw, false);
+    slab_tile<GEOM, FLAT, 1, TX, TY, TZ, true>(TA, blockIdx.x / parts, gridDim.x / parts, smem_raw, false,
+                                               blockIdx.x % parts, parts);
 }
 
-using SlabKernel = void (*)(TiledArgs<float>);
+using SlabKernel = void (*)(TiledArgs<float>, int);
 
 // The step kernel's copy for this tile shape (slab_shape_id).
 template <int GEOM, int FLAT, int MODE>
 SlabKernel step_slab_pick(int shape)
 {
-    if constexpr (MODE == 1 && FLAT == 0) {
-        if (shape == SHAPE_8C) return step_slab_kernel<GEOM, FLAT, MODE, 8, 8, 8>;
-    } else if constexpr (MODE == 1 && FLAT == 1) {
+    if constexpr (MODE == 1 && FLAT == 1) {
         if (shape == SHAPE_32X16) return step_slab_kernel<GEOM, FLAT, MODE, 32, 1, 16>;
         if (shape == SHAPE_16X16) return step_slab_kernel<GEOM, FLAT, MODE, 16, 1, 16>;
     }
@@ -1227,31 +1215,39 @@ inline size_t slab_smem_bytes(const GridDev &g)
 template <int GEOM, int FLAT, int MODE>
 cudaError_t launch_step_slab(const TiledArgs<float> &a, cudaStream_t s)
 {
-    const GridDev &g = a.s.g;
-    const int ntiles = g.nt[0] * g.nt[1] * g.nt[2];
-    const size_t smem = slab_smem_bytes(g);
-    // the default tiles (TSC, exponential midpoint) run copies compiled for
-    // their shape
-    const SlabKernel kern = step_slab_pick<GEOM, FLAT, MODE>(slab_shape_id(g, FLAT, a.tsc, MODE));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<ntiles, kSlabThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    if constexpr (FLAT == 0) {
+        return launch_cube<GEOM, MODE, false>(a, s);
+    } else {
+        const GridDev &g = a.s.g;
+        const int ntiles = g.nt[0] * g.nt[1] * g.nt[2];
+        const size_t smem = slab_smem_bytes(g);
+        // the default tiles (TSC, exponential midpoint) run copies compiled for
+        // their shape
+        const SlabKernel kern = step_slab_pick<GEOM, FLAT, MODE>(slab_shape_id(g, FLAT, a.tsc, MODE));
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int parts = tile_parts(ntiles, a.s.s.n, g.tvol, 10.0, 0.03, 0.03);
+        kern<<<ntiles * parts, kSlabThreads, smem, s>>>(a, parts);
+        return cudaGetLastError();
+    }
 }
 
 template <int GEOM, int FLAT>
 cudaError_t launch_predict_slab(const TiledArgs<float> &a, cudaStream_t s)
 {
-    const GridDev &g = a.s.g;
-    const int ntiles = g.nt[0] * g.nt[1] * g.nt[2];
-    const size_t smem = slab_smem_bytes(g);
-    SlabKernel kern = predict_slab_kernel<GEOM, FLAT>;
-    if constexpr (FLAT == 0)
-        if (slab_shape_id(g, FLAT, a.tsc, 1) == SHAPE_8C) kern = predict_slab_kernel<GEOM, FLAT, 8, 8, 8>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<ntiles, kSlabThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    if constexpr (FLAT == 0) {
+        return launch_cube<GEOM, 1, true>(a, s);
+    } else {
+        const GridDev &g = a.s.g;
+        const int ntiles = g.nt[0] * g.nt[1] * g.nt[2];
+        const size_t smem = slab_smem_bytes(g);
+        auto kern = predict_slab_kernel<GEOM, FLAT>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int parts = tile_parts(ntiles, a.s.s.n, g.tvol, 10.0, 0.03, 0.03);
+        kern<<<ntiles * parts, kSlabThreads, smem, s>>>(a, parts);
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace dust
