@@ -86,6 +86,7 @@ struct dust_ctx {
     // key counts for the next sort (d_count holds the current key offsets)
     int32_t *d_count_next = nullptr;
     bool keys_ready = false;   // d_key / d_count_next predicted by the last step
+    bool count_next_zero = false;  // d_count_next cleared by the last sort, not yet counted into
     double keys_dt = 0.0;      // the step length they were predicted for
     // steps replayed from a captured graph read their time from the device:
     // d_time = [t, shift_mid, shift_end, -]
@@ -763,7 +764,7 @@ int run_sort(dust_ctx *ctx, double dt, bool fused)
     // keys predicted by the previous step for this dt are reused; otherwise
     // the key kernel computes them
     const bool reuse = ctx->keys_ready && ctx->keys_dt == dt;
-    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_SORT] += (reuse ? 7 : 8) - (fused ? 1 : 0);
+    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_SORT] += (reuse ? 6 : 7) - (fused ? 1 : 0) + (m > scan_direct_counts() ? 1 : 0);
     if (!reuse) {
         CU(cudaMemsetAsync(ctx->d_count_next, 0, m * sizeof(int32_t), ctx->stream));
         cudaError_t e = cudaSuccess;
@@ -775,10 +776,10 @@ int run_sort(dust_ctx *ctx, double dt, bool fused)
         }
         CU(e);
     }
-    CU(launch_exclusive_scan(ctx->d_count_next, m, ctx->d_blocksums, ctx->stream));
-    CU(cudaMemcpyAsync(ctx->d_cursor, ctx->d_count_next, m * sizeof(int32_t),
-                       cudaMemcpyDeviceToDevice, ctx->stream));
-    CU(cudaMemsetAsync(ctx->d_bigseg, 0, sizeof(int32_t), ctx->stream));
+    // the buffer of the last sort's offsets receives the next counts: cleared here
+    CU(launch_exclusive_scan(ctx->d_count_next, m, ctx->d_blocksums, ctx->d_cursor, ctx->d_bigseg, ctx->d_count,
+                             ctx->stream));
+    ctx->count_next_zero = true;
     CU(launch_sort_scatter<Real>(a, ctx->stream, !fused));
     // fused: the step kernel moves the grains (and then flips the store)
     if (fused) ctx->perm_pending = true;
@@ -969,11 +970,9 @@ int run_predictor_sort(dust_ctx *ctx)
     default: e = launch_zone_keys<GEOM_SPH>(a, ctx->stream); break;
     }
     CU(e);
-    CU(launch_exclusive_scan(ctx->d_pcount, m, ctx->d_blocksums, ctx->stream));
-    CU(cudaMemcpyAsync(ctx->d_cursor, ctx->d_pcount, m * sizeof(int32_t), cudaMemcpyDeviceToDevice, ctx->stream));
-    CU(cudaMemsetAsync(ctx->d_bigseg, 0, sizeof(int32_t), ctx->stream));
+    CU(launch_exclusive_scan(ctx->d_pcount, m, ctx->d_blocksums, ctx->d_cursor, ctx->d_bigseg, nullptr, ctx->stream));
     CU(launch_sort_scatter<float>(a, ctx->stream, false));
-    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_OTHER] += 7;
+    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_OTHER] += 6 + (m > scan_direct_counts() ? 1 : 0);
     return DUST_OK;
 }
 
@@ -1077,8 +1076,9 @@ int run_step(dust_ctx *ctx, double dt)
     const int32_t *perm = pend ? ctx->d_pair_src : nullptr;
     const int32_t *perm_id = pend ? ctx->d_pair_id : nullptr;
     const StoreDev<Real> dst = store_of<Real>(ctx, 1 - ctx->cur);
-    if (emit)
+    if (emit && !ctx->count_next_zero)
         CU(cudaMemsetAsync(ctx->d_count_next, 0, (ctx->g.nkeys + 2) * sizeof(int32_t), st));
+    if (emit) ctx->count_next_zero = false;
     // tensor map of the gas the step gathers from (the predicted gas or the
     // gas at t^n)
     const int tslot = ctx->opt.gas_predictor ? 1 : 0;
@@ -1979,6 +1979,7 @@ int prime_keys(dust_ctx *ctx, double dt)
     a.tmp_id = ctx->d_key;
     a.tmp_src = ctx->d_id[1 - ctx->cur];
     CU(cudaMemsetAsync(ctx->d_count_next, 0, (ctx->g.nkeys + 2) * sizeof(int32_t), ctx->stream));
+    ctx->count_next_zero = false;
     cudaError_t e;
     switch (ctx->geom.kind) {
     case DUST_CARTESIAN: e = launch_sort_keys<Real, GEOM_CART>(a, ctx->stream); break;
@@ -2297,6 +2298,7 @@ int step_persistent(dust_batch *b, const double *dt, int nsteps)
             std::swap(c->d_count, c->d_count_next);
         }
         c->keys_ready = (nsteps % K) == 0 && c->n_grains > 0;
+        c->count_next_zero = false;
         c->keys_dt = dt[i];
         c->perm_pending = false;
         for (int s = 0; s < nsteps; ++s) c->t += dt[i];
@@ -2420,6 +2422,7 @@ extern "C" int dust_batch_step(dust_batch *b, const double *dt, int nsteps)
             for (int s = 0; s < 2 * pairs; ++s) c->t += dt[i];
             c->last_dt = dt[i];
             c->steps += 2 * pairs;
+            c->count_next_zero = false;
             c->timed_steps += 2 * pairs;
             c->have_deposit = true;
             c->need_sort = false;

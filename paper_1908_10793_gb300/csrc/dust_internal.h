@@ -344,8 +344,12 @@ cudaError_t launch_deposit_mass(const GridDev &g, const SpeciesDev &sp, int wk, 
 template <typename Real>
 cudaError_t launch_sort_scatter(const SortArgs<Real> &a, cudaStream_t s, bool gather);
 
-cudaError_t launch_exclusive_scan(int32_t *data, int64_t n, int32_t *block_sums,
-                                  cudaStream_t s);
+// Exclusive scan of data [n], the offsets copied to copy; big[0] = 0; zero
+// [n], if given, set to 0.
+cudaError_t launch_exclusive_scan(int32_t *data, int64_t n, int32_t *block_sums, int32_t *copy, int32_t *big,
+                                  int32_t *zero, cudaStream_t s);
 int64_t scan_block_sums_size(int64_t n);
+// counts beyond which the scan takes a third kernel
+int64_t scan_direct_counts();
 
 }  // namespace dust

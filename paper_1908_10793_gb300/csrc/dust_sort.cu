@@ -12,10 +12,10 @@ namespace dust {
 // chunk sums for chunks of at least 256 threads x kScanItems counts
 int64_t scan_block_sums_size(int64_t n) { return (n + 256 * kScanItems - 1) / (256 * kScanItems) + 1; }
 
-__global__ void scan_reduce_kernel(const int32_t *data, int64_t n, int32_t *block_sums)
+__global__ void scan_reduce_kernel(const int32_t *data, int64_t n, int32_t *block_sums, int32_t *zero)
 {
     __shared__ int32_t ws[32];
-    scan_reduce_block(data, n, block_sums, blockIdx.x, ws);
+    scan_reduce_block(data, n, block_sums, blockIdx.x, ws, zero);
 }
 
 __global__ void scan_sums_kernel(int32_t *block_sums, int64_t nb)
@@ -24,19 +24,33 @@ __global__ void scan_sums_kernel(int32_t *block_sums, int64_t nb)
     scan_sums_block(block_sums, nb, ws);
 }
 
-__global__ void scan_apply_kernel(int32_t *data, int64_t n, const int32_t *block_sums)
+// sums_scanned: the chunk sums are already an exclusive scan.
+__global__ void scan_finish_kernel(int32_t *data, int64_t n, const int32_t *block_sums, int sums_scanned, int32_t *copy,
+                                   int32_t *big)
 {
     __shared__ int32_t ws[32];
-    scan_apply_block(data, n, block_sums, blockIdx.x, ws, nullptr);
+    if (sums_scanned) scan_apply_block(data, n, block_sums, blockIdx.x, ws, copy);
+    else scan_finish_block(data, n, block_sums, blockIdx.x, ws, copy);
+    if (blockIdx.x == 0 && threadIdx.x == 0) big[0] = 0;
 }
 
-cudaError_t launch_exclusive_scan(int32_t *data, int64_t n, int32_t *block_sums, cudaStream_t s)
+// Up to kScanDirect chunks, each block of the second kernel sums the chunk sums
+// before it; beyond (a grid of more than 4M keys) that costs more than a
+// kernel between the two that scans them.  The copy to the cursors, the clearing of
+// the block sort's list and of the next counts are part of the two: they were a
+// copy and two clears of their own (64^2 box: sort and clears 35.7 -> 27.3 us).
+constexpr int64_t kScanDirect = 1024;
+
+int64_t scan_direct_counts() { return kScanDirect * kScanTile; }
+
+cudaError_t launch_exclusive_scan(int32_t *data, int64_t n, int32_t *block_sums, int32_t *copy, int32_t *big,
+                                  int32_t *zero, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
-    scan_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, block_sums);
-    scan_sums_kernel<<<1, kScanThreads, 0, s>>>(block_sums, nb);
-    scan_apply_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, block_sums);
+    scan_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, block_sums, zero);
+    if (nb > kScanDirect) scan_sums_kernel<<<1, kScanThreads, 0, s>>>(block_sums, nb);
+    scan_finish_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, block_sums, nb > kScanDirect, copy, big);
     return cudaGetLastError();
 }
 

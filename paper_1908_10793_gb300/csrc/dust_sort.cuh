@@ -45,15 +45,23 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *warp
 // The scan in three phases over chunks of blockDim.x * kScanItems counts
 // (device functions of a virtual block index, so that the batched
 // persistent kernel runs the same code).
-// Phase 1: sum of chunk vb.
+// Phase 1: sum of chunk vb; zero, if given, is set to 0 (the next counts).
 __device__ __forceinline__ void scan_reduce_block(const int32_t *data, int64_t n, int32_t *block_sums,
-                                                  int64_t vb, int32_t *ws)
+                                                  int64_t vb, int32_t *ws, int32_t *zero = nullptr)
 {
     const int64_t base = (vb * blockDim.x + threadIdx.x) * kScanItems;
     int32_t s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k)
-        if (base + k < n) s += data[base + k];
+    if (base + kScanItems <= n) {  // the arrays are allocations of their own: 16-byte aligned
+        const int4 x = *reinterpret_cast<const int4 *>(data + base);
+        s = x.x + x.y + x.z + x.w;
+        if (zero) *reinterpret_cast<int4 *>(zero + base) = make_int4(0, 0, 0, 0);
+    } else {
+        for (int k = 0; k < kScanItems; ++k)
+            if (base + k < n) {
+                s += data[base + k];
+                if (zero) zero[base + k] = 0;
+            }
+    }
     int32_t total;
     block_exclusive_scan(s, ws, total);
     if (threadIdx.x == 0) block_sums[vb] = total;
@@ -74,29 +82,52 @@ __device__ __forceinline__ void scan_sums_block(int32_t *block_sums, int64_t nb,
     }
 }
 
-// Phase 3: exclusive scan inside chunk vb plus the chunk's offset; copy, if
+// The chunk's counts replaced by their exclusive scan from `from`; copy, if
 // given, receives the same offsets (the scatter's cursors).
+__device__ __forceinline__ void scan_chunk(int32_t *data, int64_t n, int32_t from, int64_t vb, int32_t *ws, int32_t *copy)
+{
+    static_assert(kScanItems == 4, "one 16-byte load per thread");
+    const int64_t base = (vb * blockDim.x + threadIdx.x) * kScanItems;
+    const bool whole = base + kScanItems <= n;
+    int4 v = make_int4(0, 0, 0, 0);
+    if (whole) {
+        v = *reinterpret_cast<const int4 *>(data + base);
+    } else {
+        if (base < n) v.x = data[base];
+        if (base + 1 < n) v.y = data[base + 1];
+        if (base + 2 < n) v.z = data[base + 2];
+    }
+    int32_t total;
+    const int32_t r0 = from + block_exclusive_scan(v.x + v.y + v.z + v.w, ws, total);
+    const int4 o = make_int4(r0, r0 + v.x, r0 + v.x + v.y, r0 + v.x + v.y + v.z);
+    if (whole) {
+        *reinterpret_cast<int4 *>(data + base) = o;
+        if (copy) *reinterpret_cast<int4 *>(copy + base) = o;
+        return;
+    }
+    for (int k = 0; k < kScanItems && base + k < n; ++k) {
+        const int32_t x = k == 0 ? o.x : (k == 1 ? o.y : o.z);
+        data[base + k] = x;
+        if (copy) copy[base + k] = x;
+    }
+}
+
+// Phase 3: exclusive scan inside chunk vb plus the chunk's offset.
 __device__ __forceinline__ void scan_apply_block(int32_t *data, int64_t n, const int32_t *block_sums,
                                                  int64_t vb, int32_t *ws, int32_t *copy)
 {
-    const int64_t base = (vb * blockDim.x + threadIdx.x) * kScanItems;
-    int32_t v[kScanItems];
-    int32_t s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        v[k] = base + k < n ? data[base + k] : 0;
-        s += v[k];
-    }
-    int32_t total;
-    int32_t run = block_exclusive_scan(s, ws, total) + block_sums[vb];
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        if (base + k < n) {
-            data[base + k] = run;
-            if (copy) copy[base + k] = run;
-        }
-        run += v[k];
-    }
+    scan_chunk(data, n, block_sums[vb], vb, ws, copy);
+}
+
+// Phases 2 and 3 in one: chunk vb, whose offset the block sums from the chunk
+// sums before it, instead of a kernel between the two that scans them.
+__device__ __forceinline__ void scan_finish_block(int32_t *data, int64_t n, const int32_t *block_sums, int64_t vb,
+                                                  int32_t *ws, int32_t *copy)
+{
+    int32_t before = 0, total;
+    for (int64_t i = threadIdx.x; i < vb; i += blockDim.x) before += block_sums[i];
+    block_exclusive_scan(before, ws, total);  // total: the chunk's offset
+    scan_chunk(data, n, total, vb, ws, copy);
 }
 
 // Scatter of (id, source position) pairs to their key segments.  Positions
@@ -149,53 +180,23 @@ __device__ __forceinline__ void scatter_pairs_block(const SA &A, int64_t vb)
 // Sort by id of the (id, source) pairs of every key.  A warp takes 32
 // consecutive keys; their segments are contiguous, so the warp stages them
 // in shared memory with coalesced loads, places each pair by its rank in its
-// key's segment there, and writes them back.  When the warp's
-// segments hold more than kSegStage pairs in total, segments of at most
-// kSmallSeg pairs are insertion-sorted in place in global memory (bounded
-// cost) and longer ones are listed for the block sort below.
+// key's segment there, and writes them back.  When the warp's segments hold
+// more than kSegStage pairs in total, it takes as many keys at a time as fit;
+// a segment of more than kLongSeg pairs (whose ranks cost its length squared)
+// is then listed for the block sort below.
 constexpr int kSegThreads = 256;
 constexpr int kSegStage = 512;  // pairs staged per warp
-constexpr int kSmallSeg = 32;
+constexpr int kLongSeg = 64;
 
-__device__ __forceinline__ void insertion_sort_pairs(int32_t *id, int32_t *src, int32_t b, int32_t e)
-{
-    for (int32_t u = b + 1; u < e; ++u) {
-        const int32_t x = id[u], y = src[u];
-        int32_t j = u - 1;
-        while (j >= b) {
-            const int32_t idj = id[j];
-            if (idj <= x) break;
-            id[j + 1] = idj;
-            src[j + 1] = src[j];
-            --j;
-        }
-        id[j + 1] = x;
-        src[j + 1] = y;
-    }
-}
-
-// sid / ssrc: kSegStage pairs per warp of the block, in shared memory
+// One staging of a warp: the pairs [W0, W1) (at most kSegStage) of whole keys;
+// this lane's key holds [b, e) (b == e == W1: none of them).  sid / ssrc: the
+// warp's staging.
 template <class SA>
-__device__ __forceinline__ void segments_block(const SA &A, int64_t vb, int32_t (*sid)[kSegStage],
-                                               int32_t (*ssrc)[kSegStage])
+__device__ __forceinline__ void sort_staged(const SA &A, int32_t W0, int32_t W1, int32_t b, int32_t e, int32_t *sid,
+                                            int32_t *ssrc)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t k = vb * blockDim.x + threadIdx.x;
-    const int64_t k0 = k - lane;
-    // keys 0 .. nsort - 1 are zones; key nsort (removed grains) is left as
-    // the scatter placed it
-    const int64_t nsort = A.nkeys1 - 1;
-    if (k0 >= nsort) return;  // whole warp past the zone keys
-    const int64_t klast = min(k0 + 32, nsort);  // one past the warp's last key
-    const int32_t W0 = A.count[k0], W1 = A.count[klast];
-    const bool mine = k < nsort;
-    const int32_t b = mine ? A.count[k] : W1, e = mine ? A.count[k + 1] : W1;
-    if (W1 - W0 > kSegStage) {
-        if (mine && e - b <= kSmallSeg) insertion_sort_pairs(A.pair_id, A.pair_src, b, e);
-        else if (mine) A.big[1 + atomicAdd(&A.big[0], 1)] = (int32_t)k;
-        return;
-    }
     const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
     // all loads of a half first, then its shared stores: the loads' round
     // trips overlap
     constexpr int kHalf = kSegStage / 64;
@@ -214,20 +215,20 @@ __device__ __forceinline__ void segments_block(const SA &A, int64_t vb, int32_t 
         for (int r = 0; r < kHalf; ++r) {
             const int32_t u = W0 + lane + 32 * (r + h * kHalf);
             if (u < W1) {
-                sid[warp][u - W0] = rid[r];
-                ssrc[warp][u - W0] = rsrc[r];
+                sid[u - W0] = rid[r];
+                ssrc[u - W0] = rsrc[r];
             }
         }
     }
     __syncwarp(FULL);
     // each staged pair goes straight to its place in its key's segment: the
     // segment is found by a binary search over the lanes' segment starts
-    // (nondecreasing; lanes past the zone keys hold the end), and the place
+    // (nondecreasing; lanes without a key here hold the end), and the place
     // is the segment start plus the number of smaller ids in the segment (ids
     // are unique); the loads of the count are independent, unlike an
     // insertion sort's
     const int32_t n = W1 - W0;
-    const int32_t st = (mine ? b : W1) - W0, en = (mine ? e : W1) - W0;
+    const int32_t st = b - W0, en = e - W0;
     for (int32_t r0 = 0; r0 < n; r0 += 32) {
         const int32_t u = r0 + lane;
         int lo = 0, hi = 32;  // the last lane whose segment starts at or before u
@@ -239,12 +240,64 @@ __device__ __forceinline__ void segments_block(const SA &A, int64_t vb, int32_t 
         }
         const int32_t sb = __shfl_sync(FULL, st, lo), se = __shfl_sync(FULL, en, lo);
         if (u < n) {
-            const int32_t x = sid[warp][u];
+            const int32_t x = sid[u];
             int32_t rank = 0;
-            for (int32_t v = sb; v < se; ++v) rank += sid[warp][v] < x ? 1 : 0;
+            for (int32_t v = sb; v < se; ++v) rank += sid[v] < x ? 1 : 0;
             A.pair_id[W0 + sb + rank] = x;
-            A.pair_src[W0 + sb + rank] = ssrc[warp][u];
+            A.pair_src[W0 + sb + rank] = ssrc[u];
         }
+    }
+}
+
+// sid / ssrc: kSegStage pairs per warp of the block, in shared memory
+template <class SA>
+__device__ __forceinline__ void segments_block(const SA &A, int64_t vb, int32_t (*sid)[kSegStage],
+                                               int32_t (*ssrc)[kSegStage])
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t k = vb * blockDim.x + threadIdx.x;
+    const int64_t k0 = k - lane;
+    // keys 0 .. nsort - 1 are zones; key nsort (removed grains) is left as
+    // the scatter placed it
+    const int64_t nsort = A.nkeys1 - 1;
+    if (k0 >= nsort) return;  // whole warp past the zone keys
+    const int64_t klast = min(k0 + 32, nsort);  // one past the warp's last key
+    const int32_t W0 = A.count[k0], W1 = A.count[klast];
+    const bool mine = k < nsort;
+    const int32_t b = mine ? A.count[k] : W1, e = mine ? A.count[k + 1] : W1;
+    if (W1 - W0 <= kSegStage) {
+        sort_staged(A, W0, W1, b, e, sid[warp], ssrc[warp]);
+        return;
+    }
+    // dense zones: as many whole keys at a time as the staging holds (a disk's
+    // midplane holds more than 16 grains per zone; sorting such segments in place
+    // in global memory made the 33M-grain spherical disk's sort 965 instead of
+    // 580 us); a long key is listed for the block sort
+    int done = 0;  // keys of the warp before this lane index are finished
+    while (done < 32) {
+        const int32_t f = __shfl_sync(FULL, b, done);  // start of the first unfinished key
+        // the keys up to the first long one that end within the staging from f: a
+        // prefix of the unfinished
+        const unsigned stop = __ballot_sync(FULL, lane >= done && (e - f > kSegStage || e - b > kLongSeg));
+        const int m = stop ? __ffs(stop) - 1 : 32;
+        if (m == done) {
+            if (lane == done) A.big[1 + atomicAdd(&A.big[0], 1)] = (int32_t)k;
+            ++done;
+            continue;
+        }
+        const int32_t g = __shfl_sync(FULL, e, m - 1);  // their end
+        if (g > f) {
+            // lanes before `done` hold starts at or before f: they must not be
+            // found by the search, so every lane outside holds the end, and the
+            // keys are moved to the first lanes
+            const int from = lane + done;
+            const int32_t bb = __shfl_sync(FULL, b, from & 31), ee = __shfl_sync(FULL, e, from & 31);
+            const bool ok = from < m;
+            sort_staged(A, f, g, ok ? bb : g, ok ? ee : g, sid[warp], ssrc[warp]);
+            __syncwarp(FULL);
+        }
+        done = m;
     }
 }
 
