@@ -51,7 +51,7 @@ __device__ __forceinline__ void cube_w_cyl(int tsc, float d, float nu, float w[3
     }
 }
 
-// EXACT: as the path of grains outside their key zone rounds the CIC host weight
+// EXACT: as the path of grains outside their key zone rounds the CIC weights
 template <bool EXACT>
 __device__ __forceinline__ void cube_w_sphr(int tsc, float d, float nu, float w[3])
 {
@@ -70,7 +70,7 @@ __device__ __forceinline__ void cube_w_sphr(int tsc, float d, float nu, float w[
     } else {
         const float inv = fd(1.f, ff(fm(12.f, s), s, 1.f));
         const float ad = fabsf(d);
-        const float base = ff(2.f, d, fm(3.f, nu));
+        const float base = EXACT ? ff(2.f, d, fm(3.f, nu)) : ff(3.f, nu, fm(2.f, d));
         const float p = fa(base, 1.5f), m = fs(base, 1.5f);
         const float np_ = fa(nu, 0.5f), nm = fs(nu, 0.5f);
         const float t = ff(2.f, nu, d), u = fs(ad, 1.f);
