@@ -23,7 +23,33 @@ __device__ __forceinline__ double rcos(double x) { return cos(x); }
 __device__ __forceinline__ float rsqrt_(float x) { return sqrtf(x); }
 __device__ __forceinline__ double rsqrt_(double x) { return sqrt(x); }
 __device__ __forceinline__ long long rround(float x) { return __float2ll_rn(x); }
-__device__ __forceinline__ long long rround(double x) { return __double2ll_rn(x); }
+
+// rint(x * 2^scale) of a double below 2^51 in size after the scaling, from its
+// bit fields: the double-precision unit, which the conversion instruction
+// occupies as long as an addition (a warp instruction every ~64 cycles), bounds
+// every kernel that rounds doubles, and the integer pipe is idle there.
+__device__ __forceinline__ long long round_bits(double x, int scale)
+{
+    const long long b = __double_as_longlong(x);
+    const int s = 1075 - (int)((b >> 52) & 0x7ff) - scale;  // places the mantissa is shifted right
+    const long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+    // round half to even; more than 53 places: below one half (and zero)
+    long long v = 0;
+    if (s > 0) {
+        if (s <= 53) v = (m + ((1ll << (s - 1)) - 1) + ((m >> s) & 1)) >> s;
+    } else {
+        v = m << -s;
+    }
+    return b < 0 ? -v : v;
+}
+
+// The same integer as __double2ll_rn.
+__device__ __forceinline__ long long rround(double x)
+{
+    // exponents from 2^51 on (and NaN) take the instruction
+    if (((__double_as_longlong(x) >> 52) & 0x7ff) >= 1023 + 51) return __double2ll_rn(x);
+    return round_bits(x, 0);
+}
 
 // Shear-periodic shifts of the step at its half and full time: from the
 // kernel arguments, or from device memory for steps replayed from a graph.

@@ -8,6 +8,63 @@ namespace dust {
 
 constexpr int kStepThreads = 256;
 
+// |x| < 4.5e15 (false for NaN): a deposit piece or sum in range.  In double
+// precision by the bit pattern, on the integer pipe: the double-precision pipe
+// bounds the FP64 kernels.
+__device__ __forceinline__ bool in_range(float x) { return fabsf(x) < 4.5e15f; }
+__device__ __forceinline__ bool in_range(double x)
+{
+    return (__double_as_longlong(x) & 0x7fffffffffffffffll) < 0x432ff973cafa8000ll;  // the bits of 4.5e15
+}
+
+// NaN and finiteness tests by the bit pattern.
+__device__ __forceinline__ bool bits_nan(double x)
+{
+    return (__double_as_longlong(x) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool bits_finite(float x) { return isfinite(x); }
+__device__ __forceinline__ bool bits_finite(double x)
+{
+    return (__double_as_longlong(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
+}
+
+// Stopping time and propagators (Eqs. phi1, h1) of the species whose grains all
+// have the same stopping time (constant tau; constant Stokes number in
+// Cartesian and shearing-box geometry), evaluated once per block with the same
+// operations as per grain, so the bits are the same.  A grain's two divisions,
+// exp and expm1 were a seventh of the FP64 tiled step's double-precision
+// operations.
+template <typename Real>
+struct Propagators {
+    Real tau[kMaxSpecies], E[kMaxSpecies], cg[kMaxSpecies], h1[kMaxSpecies];
+};
+
+template <int GEOM>
+__device__ __forceinline__ bool tau_is_shared(int mode)
+{
+    return mode == DUST_TAU_CONST || (mode == DUST_TAU_STOKES && (GEOM == GEOM_CART || GEOM == GEOM_SB));
+}
+
+template <typename Real>
+__device__ __forceinline__ void propagate(Real tau, Real dt, Real &E, Real &cg, Real &h1)
+{
+    const Real x = dt / tau;
+    E = rexp(-x);
+    cg = -rexpm1(-x);
+    h1 = (x == Real(0)) ? dt : dt * cg / x;
+}
+
+// Every thread of the block calls it; a block barrier must follow.
+template <typename Real, int GEOM>
+__device__ __forceinline__ void shared_propagators(const StepArgs<Real> &A, Propagators<Real> &P)
+{
+    const int k = threadIdx.x;
+    if (A.s.param || k >= A.sp.n || !tau_is_shared<GEOM>(A.sp.mode[k])) return;
+    const double none[3] = {0.0, 0.0, 0.0};
+    P.tau[k] = stopping_time<Real, GEOM>(A.ph, A.sp.mode[k], (Real)A.sp.tau[k], none, Real(1));
+    propagate<Real>(P.tau[k], (Real)A.dt, P.E[k], P.cg[k], P.h1[k]);
+}
+
 // Per-grain fixed-point deposit rule: for every channel c the grain's total
 // Q_c = rint(D_c / quantum) is split over the stencil; every node other than
 // the host gets rint(W_j D_c / quantum) and the host gets the remainder, so
@@ -22,7 +79,7 @@ __device__ __forceinline__ void deposit_fixed(const GridDev &g, unsigned long lo
     bool big = false;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        big |= !(fabs(Dq[c]) < Real(4.5e15));  // in the working precision
+        big |= !in_range(Dq[c]);
         rest[c] = rround(Dq[c]);
     }
     if (big) atomicOr(&status[ST_FLAGS], DUST_FLAG_OVERFLOW);
@@ -89,6 +146,9 @@ __global__ void __launch_bounds__(kStepThreads)
 step_per_grain_kernel(const StepArgs<Real> A)
 {
     const int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ Propagators<Real> prop;
+    shared_propagators<Real, GEOM>(A, prop);
+    __syncthreads();
     bool removed = false;
     float moved = 0.f;
     if (gi < A.s.n) {
@@ -97,8 +157,8 @@ step_per_grain_kernel(const StepArgs<Real> A)
         // a species index the species table does not hold (possible only
         // where the caller owns the store): flagged, the grain left as it is
         const bool sp_ok = sp < A.sp.n;
-        if (!sp_ok && !isnan(q[0])) atomicOr(&A.status[ST_FLAGS], DUST_FLAG_SPECIES);
-        if (!isnan(q[0]) && sp_ok) {
+        if (!sp_ok && !bits_nan(q[0])) atomicOr(&A.status[ST_FLAGS], DUST_FLAG_SPECIES);
+        if (!bits_nan(q[0]) && sp_ok) {
             Real pn[3] = {A.s.p[0][gi], A.s.p[1][gi], A.s.p[2][gi]};
             const Real h = (Real)(0.5 * A.dt);
             Real inc1[3], inc2[3];
@@ -137,13 +197,18 @@ step_per_grain_kernel(const StepArgs<Real> A)
                         }
                     }
                 }
-                const Real value = A.s.param ? A.s.param[gi] : (Real)A.sp.tau[sp];
-                const Real tau = stopping_time<Real, GEOM>(A.ph, A.sp.mode[sp], value, qm, acc[0]);
                 const Real dt = (Real)A.dt;
-                const Real x = dt / tau;
-                const Real E = rexp(-x);
-                const Real cg = -rexpm1(-x);
-                const Real h1 = (x == Real(0)) ? dt : dt * cg / x;
+                Real tau, E, cg, h1;
+                if (!A.s.param && tau_is_shared<GEOM>(A.sp.mode[sp])) {
+                    tau = prop.tau[sp];
+                    E = prop.E[sp];
+                    cg = prop.cg[sp];
+                    h1 = prop.h1[sp];
+                } else {
+                    const Real value = A.s.param ? A.s.param[gi] : (Real)A.sp.tau[sp];
+                    tau = stopping_time<Real, GEOM>(A.ph, A.sp.mode[sp], value, qm, acc[0]);
+                    propagate<Real>(tau, dt, E, cg, h1);
+                }
                 const Real vg[3] = {acc[1], acc[2], acc[3]};
                 Real pp[3], a[3], dH[3];
                 kick_any<Real, GEOM>(A.ph, qm, pn, vg, tau, dt, E, cg, h1, pp, a, dH);
@@ -160,7 +225,7 @@ step_per_grain_kernel(const StepArgs<Real> A)
                     Dq[3] += Dq[c] * dH[c];
                 }
                 deposit_fixed<Real>(A.g, A.dep, host, w, Dq, A.status);
-                if (!(isfinite(pp[0]) && isfinite(pp[1]) && isfinite(pp[2])))
+                if (!(bits_finite(pp[0]) && bits_finite(pp[1]) && bits_finite(pp[2])))
                     atomicOr(&A.status[ST_FLAGS], DUST_FLAG_NAN);
 #pragma unroll
                 for (int d = 0; d < 3; ++d)
@@ -172,7 +237,7 @@ step_per_grain_kernel(const StepArgs<Real> A)
                 A.s.q[0][gi] = q[0]; A.s.q[1][gi] = q[1]; A.s.q[2][gi] = q[2];
                 A.s.p[0][gi] = pnew[0]; A.s.p[1][gi] = pnew[1]; A.s.p[2][gi] = pnew[2];
             }
-            if (removed && !(isnan(A.s.q[0][gi]))) A.s.q[0][gi] = __longlong_as_double(0x7ff8000000000000LL);
+            if (removed && !bits_nan(A.s.q[0][gi])) A.s.q[0][gi] = __longlong_as_double(0x7ff8000000000000LL);
         }
     }
     // warp-aggregated status updates
@@ -328,25 +393,43 @@ __global__ void deposit_mass_kernel(GridDev g, SpeciesDev sp, int wk, int64_t n,
 #pragma unroll
     for (int d = 0; d < 3; ++d) zone_weights<double, GEOM>(g, d, wk, q[d], host[d], w[d], iw[d]);
     const double M = sp.mq[species ? species[k] : 0];
-    if (!(fabs(M) < 4.5e15)) atomicOr(&status[ST_FLAGS], DUST_FLAG_OVERFLOW);
+    if (!in_range(M)) atomicOr(&status[ST_FLAGS], DUST_FLAG_OVERFLOW);
     long long rest = rround(M);
-#pragma unroll 1
-    for (int nd = 0; nd < 27; ++nd) {
-        const int a = nd % 3, b = (nd / 3) % 3, c = nd / 9;
-        if (nd == 13 || (g.n[0] <= 1 && a != 1) || (g.n[1] <= 1 && b != 1) || (g.n[2] <= 1 && c != 1))
-            continue;
-        const long long piece = rround(w[0][a] * w[1][b] * w[2][c] * M);
-        if (piece == 0) continue;
-        const int ix = node_of(host[0], a - 1, g.n[0], g.bc[0]);
-        const int iy = node_of(host[1], b - 1, g.n[1], g.bc[1]);
-        const int iz = node_of(host[2], c - 1, g.n[2], g.bc[2]);
-        atomicAdd(&out[ix + (int64_t)g.n[0] * (iy + (int64_t)g.n[1] * iz)], (unsigned long long)piece);
-        rest -= piece;
+    // a power of two (every species at the default quantum that has the largest
+    // mass) scales exactly: the product with it is left to the rounding's shift
+    const long long mb = __double_as_longlong(M);
+    const int me = (int)((mb >> 52) & 0x7ff) - 1023;
+    const bool pow2 = mb > 0 && (mb & 0xfffffffffffffll) == 0 && me >= 0 && me <= 50;
+    const bool g0 = g.n[0] > 1, g1 = g.n[1] > 1, g2 = g.n[2] > 1;
+    int ix[3], iy[3], iz[3];
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+        ix[o] = node_of(host[0], o - 1, g.n[0], g.bc[0]);
+        iy[o] = node_of(host[1], o - 1, g.n[1], g.bc[1]);
+        iz[o] = node_of(host[2], o - 1, g.n[2], g.bc[2]);
     }
-    const int64_t h = node_of(host[0], 0, g.n[0], g.bc[0]) +
-                      (int64_t)g.n[0] * (node_of(host[1], 0, g.n[1], g.bc[1]) +
-                                         (int64_t)g.n[1] * node_of(host[2], 0, g.n[2], g.bc[2]));
-    if (rest != 0) atomicAdd(&out[h], (unsigned long long)rest);
+    // the product w0 w1 is formed once for the nodes that share it; unrolled, so
+    // that the weights stay in registers
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        if (!g1 && b != 1) continue;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (!g0 && a != 1) continue;
+            const double wab = w[0][a] * w[1][b];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if ((!g2 && c != 1) || (a == 1 && b == 1 && c == 1)) continue;
+                const double W = wab * w[2][c];
+                const long long piece = pow2 ? round_bits(W, me) : rround(W * M);
+                if (piece == 0) continue;
+                atomicAdd(&out[ix[a] + (int64_t)g.n[0] * (iy[b] + (int64_t)g.n[1] * iz[c])], (unsigned long long)piece);
+                rest -= piece;
+            }
+        }
+    }
+    if (rest != 0)
+        atomicAdd(&out[ix[1] + (int64_t)g.n[0] * (iy[1] + (int64_t)g.n[1] * iz[1])], (unsigned long long)rest);
 }
 
 template <int GEOM>

@@ -288,6 +288,8 @@ step_tiled_kernel(const TiledArgs<Real> TA)
         for (int c = 0; c < 4; ++c) sdep[c * bvol + lin] = 0ull;
     }
     for (int k = threadIdx.x; k < 4 * CH; k += blockDim.x) run_sum[k] = 0ull;
+    __shared__ Propagators<Real> prop;
+    shared_propagators<Real, GEOM>(A, prop);
     __syncthreads();
     if (!gas_box_finish<Real>(g, A.gas, TA.gas_tmap, sgas, o, B, sbar, A.status, TA.wait_ns)) return;
 
@@ -333,7 +335,7 @@ step_tiled_kernel(const TiledArgs<Real> TA)
         int hl = -1;
         if (slot < cn) {
             double q[3] = {A.s.q[0][gi], A.s.q[1][gi], A.s.q[2][gi]};
-            if (!isnan(q[0])) {
+            if (!bits_nan(q[0])) {
                 Real pn[3] = {A.s.p[0][gi], A.s.p[1][gi], A.s.p[2][gi]};
                 const int sp = A.s.species ? A.s.species[gi] : 0;
                 Real inc1[3], inc2[3];
@@ -388,12 +390,17 @@ step_tiled_kernel(const TiledArgs<Real> TA)
                             }
                         }
                     }
-                    const Real value = A.s.param ? A.s.param[gi] : (Real)A.sp.tau[sp];
-                    const Real tau = stopping_time<Real, GEOM>(A.ph, A.sp.mode[sp], value, qm, acc[0]);
-                    const Real x = dt / tau;
-                    const Real E = rexp(-x);
-                    const Real cg = -rexpm1(-x);
-                    const Real h1 = (x == Real(0)) ? dt : dt * cg / x;
+                    Real tau, E, cg, h1;
+                    if (!A.s.param && tau_is_shared<GEOM>(A.sp.mode[sp])) {
+                        tau = prop.tau[sp];
+                        E = prop.E[sp];
+                        cg = prop.cg[sp];
+                        h1 = prop.h1[sp];
+                    } else {
+                        const Real value = A.s.param ? A.s.param[gi] : (Real)A.sp.tau[sp];
+                        tau = stopping_time<Real, GEOM>(A.ph, A.sp.mode[sp], value, qm, acc[0]);
+                        propagate<Real>(tau, dt, E, cg, h1);
+                    }
                     const Real vg[3] = {acc[1], acc[2], acc[3]};
                     Real pp[3], a[3], dH[3];
                     kick_any<Real, GEOM>(A.ph, qm, pn, vg, tau, dt, E, cg, h1, pp, a, dH);
@@ -408,7 +415,7 @@ step_tiled_kernel(const TiledArgs<Real> TA)
                         Dq[c] = -mq * ((pp[c] - pn[c]) - dt * a[c]);
                         Dq[3] += Dq[c] * dH[c];
                     }
-                    if (!(isfinite(pp[0]) && isfinite(pp[1]) && isfinite(pp[2])))
+                    if (!(bits_finite(pp[0]) && bits_finite(pp[1]) && bits_finite(pp[2])))
                         atomicOr(&A.status[ST_FLAGS], DUST_FLAG_NAN);
 #pragma unroll
                     for (int d = 0; d < 3; ++d)
@@ -521,7 +528,7 @@ step_tiled_kernel(const TiledArgs<Real> TA)
                     const int lin = hlin + (a - 1) + B[0] * ((b - 1) + B[1] * (z - 1));
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        big |= !(fabs(sum[z][c]) < Real(4.5e15));
+                        big |= !in_range(sum[z][c]);
                         const long long piece = rround(sum[z][c]);
                         if (piece != 0) {
                             shared_add_i64(&sdep[c * bvol + lin], piece);
@@ -533,7 +540,7 @@ step_tiled_kernel(const TiledArgs<Real> TA)
                 for (int c = 0; c < 4; ++c) {
                     if (ps[c] != 0) shared_add_i64(&run_sum[c * CH + r], ps[c]);
                     if (htask) {
-                        big |= !(fabs(S[c]) < Real(4.5e15));
+                        big |= !in_range(S[c]);
                         run_q[c * CH + r] = rround(S[c]);
                     }
                 }
