@@ -86,6 +86,7 @@ struct dust_ctx {
     // key counts for the next sort (d_count holds the current key offsets)
     int32_t *d_count_next = nullptr;
     bool keys_ready = false;   // d_key / d_count_next predicted by the last step
+    bool dep_zero = false;         // d_dep cleared by the sort of the step being enqueued
     bool count_next_zero = false;  // d_count_next cleared by the last sort, not yet counted into
     double keys_dt = 0.0;      // the step length they were predicted for
     // steps replayed from a captured graph read their time from the device:
@@ -737,6 +738,9 @@ int alloc_store(dust_ctx *ctx, int64_t n)
     return DUST_OK;
 }
 
+// Deposits up to this size are cleared by the sort's scan.
+constexpr int64_t kScanClearsDeposit = 16 << 20;
+
 template <typename Real>
 int run_sort(dust_ctx *ctx, double dt, bool fused)
 {
@@ -764,7 +768,7 @@ int run_sort(dust_ctx *ctx, double dt, bool fused)
     // keys predicted by the previous step for this dt are reused; otherwise
     // the key kernel computes them
     const bool reuse = ctx->keys_ready && ctx->keys_dt == dt;
-    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_SORT] += (reuse ? 6 : 7) - (fused ? 1 : 0) + (m > scan_direct_counts() ? 1 : 0);
+    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_SORT] += (reuse ? 4 : 5) - (fused ? 1 : 0) + scan_launches(m);
     if (!reuse) {
         CU(cudaMemsetAsync(ctx->d_count_next, 0, m * sizeof(int32_t), ctx->stream));
         cudaError_t e = cudaSuccess;
@@ -776,10 +780,15 @@ int run_sort(dust_ctx *ctx, double dt, bool fused)
         }
         CU(e);
     }
-    // the buffer of the last sort's offsets receives the next counts: cleared here
+    // the buffer of the last sort's offsets receives the next counts, and the
+    // deposit the coming step's: both cleared here (a large deposit by a clear of
+    // its own: it is bound by memory either way, and the launch no longer counts)
+    const int64_t dep_bytes = ctx->ncell * 4 * (int64_t)sizeof(unsigned long long);
+    const bool clear_dep = dep_bytes <= kScanClearsDeposit;
     CU(launch_exclusive_scan(ctx->d_count_next, m, ctx->d_blocksums, ctx->d_cursor, ctx->d_bigseg, ctx->d_count,
-                             ctx->stream));
+                             clear_dep ? ctx->d_dep : nullptr, clear_dep ? dep_bytes : 0, ctx->stream));
     ctx->count_next_zero = true;
+    ctx->dep_zero = clear_dep;
     CU(launch_sort_scatter<Real>(a, ctx->stream, !fused));
     // fused: the step kernel moves the grains (and then flips the store)
     if (fused) ctx->perm_pending = true;
@@ -970,9 +979,10 @@ int run_predictor_sort(dust_ctx *ctx)
     default: e = launch_zone_keys<GEOM_SPH>(a, ctx->stream); break;
     }
     CU(e);
-    CU(launch_exclusive_scan(ctx->d_pcount, m, ctx->d_blocksums, ctx->d_cursor, ctx->d_bigseg, nullptr, ctx->stream));
+    CU(launch_exclusive_scan(ctx->d_pcount, m, ctx->d_blocksums, ctx->d_cursor, ctx->d_bigseg, nullptr, nullptr, 0,
+                             ctx->stream));
     CU(launch_sort_scatter<float>(a, ctx->stream, false));
-    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_OTHER] += 6 + (m > scan_direct_counts() ? 1 : 0);
+    if (ctx->n_grains > 0) ctx->launches[dust_ctx::GROUP_OTHER] += 4 + scan_launches(m);
     return DUST_OK;
 }
 
@@ -1008,7 +1018,9 @@ int run_step(dust_ctx *ctx, double dt)
     a.tdev = ctx->capture_mode ? ctx->d_time : nullptr;
     {
         GroupTimer timer(ctx, dust_ctx::GROUP_OTHER);
-        CU(cudaMemsetAsync(ctx->d_dep, 0, ctx->ncell * 4 * sizeof(unsigned long long), ctx->stream));
+        if (!ctx->dep_zero)
+            CU(cudaMemsetAsync(ctx->d_dep, 0, ctx->ncell * 4 * sizeof(unsigned long long), ctx->stream));
+        ctx->dep_zero = false;
         if (ctx->opt.gas_predictor) {
             // predictor: drag of the grains at x^n advances the gas by dt/2;
             // the step gathers from the prediction, the feedback corrects the

@@ -345,11 +345,14 @@ template <typename Real>
 cudaError_t launch_sort_scatter(const SortArgs<Real> &a, cudaStream_t s, bool gather);
 
 // Exclusive scan of data [n], the offsets copied to copy; big[0] = 0; zero
-// [n], if given, set to 0.
+// [n] and dep [dep_bytes] (a multiple of 16), if given, set to 0.
 cudaError_t launch_exclusive_scan(int32_t *data, int64_t n, int32_t *block_sums, int32_t *copy, int32_t *big,
-                                  int32_t *zero, cudaStream_t s);
+                                  int32_t *zero, void *dep, int64_t dep_bytes, cudaStream_t s);
 int64_t scan_block_sums_size(int64_t n);
-// counts beyond which the scan takes a third kernel
+// counts beyond which the scan takes a third kernel, and up to which it takes one
 int64_t scan_direct_counts();
+int64_t scan_small_counts();
+// kernels of a scan of m counts
+inline int scan_launches(int64_t m) { return m <= scan_small_counts() ? 1 : (m > scan_direct_counts() ? 3 : 2); }
 
 }  // namespace dust

@@ -12,10 +12,27 @@ namespace dust {
 // chunk sums for chunks of at least 256 threads x kScanItems counts
 int64_t scan_block_sums_size(int64_t n) { return (n + 256 * kScanItems - 1) / (256 * kScanItems) + 1; }
 
-__global__ void scan_reduce_kernel(const int32_t *data, int64_t n, int32_t *block_sums, int32_t *zero)
+// Buffers the scan's kernels clear on their way, so that the clears need no
+// launches of their own: the next counts (zero, as many as are scanned) and the
+// deposit of the coming step (words of 16 bytes).
+struct ScanClears {
+    int32_t *zero;
+    uint4 *dep;
+    int64_t dep_words;
+};
+
+__device__ __forceinline__ void clear_deposit(const ScanClears &C)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < C.dep_words;
+         i += (int64_t)gridDim.x * blockDim.x)
+        C.dep[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+__global__ void scan_reduce_kernel(const int32_t *data, int64_t n, int32_t *block_sums, const ScanClears C)
 {
     __shared__ int32_t ws[32];
-    scan_reduce_block(data, n, block_sums, blockIdx.x, ws, zero);
+    scan_reduce_block(data, n, block_sums, blockIdx.x, ws, C.zero);
+    clear_deposit(C);
 }
 
 __global__ void scan_sums_kernel(int32_t *block_sums, int64_t nb)
@@ -34,21 +51,41 @@ __global__ void scan_finish_kernel(int32_t *data, int64_t n, const int32_t *bloc
     if (blockIdx.x == 0 && threadIdx.x == 0) big[0] = 0;
 }
 
+// A few chunks: block 0 scans them in turn; the other blocks only clear.
+__global__ void scan_small_kernel(int32_t *data, int64_t n, int32_t *copy, int32_t *big, const ScanClears C)
+{
+    __shared__ int32_t ws[32];
+    clear_deposit(C);
+    if (blockIdx.x > 0) return;
+    int32_t from = 0;
+    for (int64_t vb = 0; vb * kScanTile < n; ++vb) from += scan_chunk(data, n, from, vb, ws, copy, C.zero);
+    if (threadIdx.x == 0) big[0] = 0;
+}
+
 // Up to kScanDirect chunks, each block of the second kernel sums the chunk sums
 // before it; beyond (a grid of more than 4M keys) that costs more than a
-// kernel between the two that scans them.  The copy to the cursors, the clearing of
-// the block sort's list and of the next counts are part of the two: they were a
-// copy and two clears of their own (64^2 box: sort and clears 35.7 -> 27.3 us).
-constexpr int64_t kScanDirect = 1024;
+// kernel between the two that scans them.  Up to kScanSmall chunks take one
+// launch.  The copy to the cursors and the clears are part of these kernels: they
+// were a copy and three clears of their own (64^2 box: sort and clears 35.7 ->
+// 27.3 us with two launches).
+constexpr int64_t kScanDirect = 1024, kScanSmall = 4;
 
 int64_t scan_direct_counts() { return kScanDirect * kScanTile; }
+int64_t scan_small_counts() { return kScanSmall * kScanTile; }
 
 cudaError_t launch_exclusive_scan(int32_t *data, int64_t n, int32_t *block_sums, int32_t *copy, int32_t *big,
-                                  int32_t *zero, cudaStream_t s)
+                                  int32_t *zero, void *dep, int64_t dep_bytes, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
-    scan_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, block_sums, zero);
+    const ScanClears C{zero, static_cast<uint4 *>(dep), dep_bytes / (int64_t)sizeof(uint4)};
+    // enough blocks to clear the deposit at the memory's rate
+    if (nb <= kScanSmall) {
+        const int64_t clears = (C.dep_words + kScanTile - 1) / kScanTile;
+        scan_small_kernel<<<(unsigned)(1 + (clears < 304 ? clears : 304)), kScanThreads, 0, s>>>(data, n, copy, big, C);
+        return cudaGetLastError();
+    }
+    scan_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, block_sums, C);
     if (nb > kScanDirect) scan_sums_kernel<<<1, kScanThreads, 0, s>>>(block_sums, nb);
     scan_finish_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, block_sums, nb > kScanDirect, copy, big);
     return cudaGetLastError();

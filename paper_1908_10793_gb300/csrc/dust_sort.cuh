@@ -83,8 +83,10 @@ __device__ __forceinline__ void scan_sums_block(int32_t *block_sums, int64_t nb,
 }
 
 // The chunk's counts replaced by their exclusive scan from `from`; copy, if
-// given, receives the same offsets (the scatter's cursors).
-__device__ __forceinline__ void scan_chunk(int32_t *data, int64_t n, int32_t from, int64_t vb, int32_t *ws, int32_t *copy)
+// given, receives the same offsets (the scatter's cursors); zero, if given, is
+// set to 0.  Returns the chunk's sum.
+__device__ __forceinline__ int32_t scan_chunk(int32_t *data, int64_t n, int32_t from, int64_t vb, int32_t *ws,
+                                              int32_t *copy, int32_t *zero = nullptr)
 {
     static_assert(kScanItems == 4, "one 16-byte load per thread");
     const int64_t base = (vb * blockDim.x + threadIdx.x) * kScanItems;
@@ -103,13 +105,16 @@ __device__ __forceinline__ void scan_chunk(int32_t *data, int64_t n, int32_t fro
     if (whole) {
         *reinterpret_cast<int4 *>(data + base) = o;
         if (copy) *reinterpret_cast<int4 *>(copy + base) = o;
-        return;
+        if (zero) *reinterpret_cast<int4 *>(zero + base) = make_int4(0, 0, 0, 0);
+        return total;
     }
     for (int k = 0; k < kScanItems && base + k < n; ++k) {
         const int32_t x = k == 0 ? o.x : (k == 1 ? o.y : o.z);
         data[base + k] = x;
         if (copy) copy[base + k] = x;
+        if (zero) zero[base + k] = 0;
     }
+    return total;
 }
 
 // Phase 3: exclusive scan inside chunk vb plus the chunk's offset.
@@ -266,35 +271,36 @@ __device__ __forceinline__ void segments_block(const SA &A, int64_t vb, int32_t 
     const int32_t W0 = A.count[k0], W1 = A.count[klast];
     const bool mine = k < nsort;
     const int32_t b = mine ? A.count[k] : W1, e = mine ? A.count[k + 1] : W1;
-    if (W1 - W0 <= kSegStage) {
-        sort_staged(A, W0, W1, b, e, sid[warp], ssrc[warp]);
-        return;
-    }
-    // dense zones: as many whole keys at a time as the staging holds (a disk's
-    // midplane holds more than 16 grains per zone; sorting such segments in place
-    // in global memory made the 33M-grain spherical disk's sort 965 instead of
-    // 580 us); a long key is listed for the block sort
-    int done = 0;  // keys of the warp before this lane index are finished
-    while (done < 32) {
-        const int32_t f = __shfl_sync(FULL, b, done);  // start of the first unfinished key
-        // the keys up to the first long one that end within the staging from f: a
-        // prefix of the unfinished
-        const unsigned stop = __ballot_sync(FULL, lane >= done && (e - f > kSegStage || e - b > kLongSeg));
-        const int m = stop ? __ffs(stop) - 1 : 32;
-        if (m == done) {
-            if (lane == done) A.big[1 + atomicAdd(&A.big[0], 1)] = (int32_t)k;
-            ++done;
-            continue;
-        }
-        const int32_t g = __shfl_sync(FULL, e, m - 1);  // their end
-        if (g > f) {
-            // lanes before `done` hold starts at or before f: they must not be
-            // found by the search, so every lane outside holds the end, and the
-            // keys are moved to the first lanes
+    // usually all 32 keys at once.  Dense zones: as many whole keys at a time as
+    // the staging holds (a disk's midplane holds more than 16 grains per zone;
+    // sorting such segments in place in global memory made the 33M-grain
+    // spherical disk's sort 965 instead of 536 us); a long key is listed for the
+    // block sort
+    const bool all = W1 - W0 <= kSegStage;
+    for (int done = 0; done < 32;) {  // keys of the warp before lane index `done` are finished
+        int m = 32;
+        int32_t f = W0, g = W1, bb = b, ee = e;
+        if (!all) {
+            f = __shfl_sync(FULL, b, done);  // start of the first unfinished key
+            // the keys up to the first long one that end within the staging from
+            // f: a prefix of the unfinished
+            const unsigned stop = __ballot_sync(FULL, lane >= done && (e - f > kSegStage || e - b > kLongSeg));
+            if (stop) m = __ffs(stop) - 1;
+            if (m == done) {
+                if (lane == done) A.big[1 + atomicAdd(&A.big[0], 1)] = (int32_t)k;
+                ++done;
+                continue;
+            }
+            g = __shfl_sync(FULL, e, m - 1);  // their end
+            // the keys are moved to the first lanes; the lanes without one hold
+            // the end, so that the search does not find them
             const int from = lane + done;
-            const int32_t bb = __shfl_sync(FULL, b, from & 31), ee = __shfl_sync(FULL, e, from & 31);
-            const bool ok = from < m;
-            sort_staged(A, f, g, ok ? bb : g, ok ? ee : g, sid[warp], ssrc[warp]);
+            bb = __shfl_sync(FULL, b, from & 31);
+            ee = __shfl_sync(FULL, e, from & 31);
+            if (from >= m) bb = ee = g;
+        }
+        if (g > f) {
+            sort_staged(A, f, g, bb, ee, sid[warp], ssrc[warp]);
             __syncwarp(FULL);
         }
         done = m;
