@@ -507,6 +507,29 @@ __device__ __forceinline__ void kick_si(const PhysDev &ph, const QT qm[3], const
 }
 
 // ---------------------------------------------------------------- kick ----
+// Sums of products of the curvilinear kicks with the roundings spelled out:
+// which product of a sum the compiler fuses depends on the code around it (with
+// E and 1 - E read from a table instead of computed in place it took the other
+// one, and a third of the velocities moved by a unit in the last place).
+__device__ __forceinline__ double fma_of(double a, double x, double y) { return __fma_rn(a, x, y); }
+__device__ __forceinline__ float fma_of(float a, float x, float y) { return __fmaf_rn(a, x, y); }
+__device__ __forceinline__ double mul_of(double a, double x) { return __dmul_rn(a, x); }
+__device__ __forceinline__ float mul_of(float a, float x) { return __fmul_rn(a, x); }
+
+// a x + b y
+template <typename Real>
+__device__ __forceinline__ Real sum2(Real a, Real x, Real b, Real y)
+{
+    return fma_of(a, x, mul_of(b, y));
+}
+
+// a x + b y + c z
+template <typename Real>
+__device__ __forceinline__ Real sum3(Real a, Real x, Real b, Real y, Real c, Real z)
+{
+    return fma_of(c, z, sum2(a, x, b, y));
+}
+
 // Kick with E = exp(-dt/tau), cg = 1 - E = h1/tau, h1 = dt phi1(-dt/tau)
 // (Eqs. phi1, h1); returns the new p, the non-frictional acceleration a at
 // (q^{n+1/2}, p^{n+1/2}) and dH/dp at the half step.
@@ -564,10 +587,10 @@ __device__ __forceinline__ void kick(const PhysDev &ph, const QT qm[3], const Re
             }
         }
         pp[2] = E * pn[2] + h1 * gz + cg * vg[2];
-        pp[1] = E * pn[1] + cg * vg[1];
-        const Real l2 = Real(0.5) * (pn[1] * pn[1] + pp[1] * pp[1]);
+        pp[1] = sum2(E, pn[1], cg, vg[1]);
+        const Real l2 = Real(0.5) * sum2(pn[1], pn[1], pp[1], pp[1]);
         const Real aR = l2 / (R * R * R) + gR;
-        pp[0] = E * pn[0] + h1 * aR + cg * vg[0];
+        pp[0] = sum3(E, pn[0], h1, aR, cg, vg[0]);
         a[0] = aR; a[1] = Real(0); a[2] = gz;
         dH[0] = Real(0.5) * (pn[0] + pp[0]);
         dH[1] = Real(0.5) * (pn[1] + pp[1]) / (R * R);
@@ -578,13 +601,13 @@ __device__ __forceinline__ void kick(const PhysDev &ph, const QT qm[3], const Re
         const Real th = (Real)qm[1];
         const Real st = rsin(th), ct = rcos(th);
         const Real gr = ph.gm != 0.0 ? -pick<Real>(ph.gm, ph.gm_f) / (r * r) : Real(0);
-        pp[2] = E * pn[2] + cg * vg[2];
-        const Real lp2 = Real(0.5) * (pn[2] * pn[2] + pp[2] * pp[2]);
+        pp[2] = sum2(E, pn[2], cg, vg[2]);
+        const Real lp2 = Real(0.5) * sum2(pn[2], pn[2], pp[2], pp[2]);
         const Real ath = lp2 * ct / (r * r * st * st * st);
-        pp[1] = E * pn[1] + h1 * ath + cg * vg[1];
-        const Real lt2 = Real(0.5) * (pn[1] * pn[1] + pp[1] * pp[1]);
+        pp[1] = sum3(E, pn[1], h1, ath, cg, vg[1]);
+        const Real lt2 = Real(0.5) * sum2(pn[1], pn[1], pp[1], pp[1]);
         const Real ar = (lt2 + lp2 / (st * st)) / (r * r * r) + gr;
-        pp[0] = E * pn[0] + h1 * ar + cg * vg[0];
+        pp[0] = sum3(E, pn[0], h1, ar, cg, vg[0]);
         a[0] = ar; a[1] = ath; a[2] = Real(0);
         dH[0] = Real(0.5) * (pn[0] + pp[0]);
         dH[1] = Real(0.5) * (pn[1] + pp[1]) / (r * r);
