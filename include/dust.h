@@ -93,8 +93,9 @@ enum { DUST_MEM_HOST = 0, DUST_MEM_DEVICE = 1 };
  * DUST_KERNEL_TILED: one block per tile of zones, gas stencil and deposit in
  * shared memory, deposit quantised once per run (grains of one zone sharing
  * their half-step host zone).  DUST_KERNEL_SLAB (mixed precision, x gridded):
- * like the tiled kernel, but three lanes own one zone and keep its stencil
- * and its deposit in registers.  DUST_KERNEL_AUTO: the slab kernel where it
+ * like the tiled kernel, but a warp pushes 32 grains at a time and keeps the
+ * deposit in registers (in 3-D a stencil node per lane, in 2-D three lanes per
+ * zone).  DUST_KERNEL_AUTO: the slab kernel where it
  * applies, else the tiled kernel. */
 enum { DUST_KERNEL_AUTO = 0, DUST_KERNEL_PER_GRAIN = 1, DUST_KERNEL_TILED = 2, DUST_KERNEL_SLAB = 3 };
 
