@@ -40,6 +40,31 @@ constexpr int kCubeThreads = 256;
 constexpr int kCubeRec = 20;
 constexpr int kCubeOne = 16;
 
+// Chunk sums below this (and the host's share) take the 32-bit rounding; the
+// host's rest, which differs from its share by rounding only, then needs that
+// rounding to stay below 1.47e8.
+constexpr float kCubeNarrow = 2e9f;
+
+// With at most kSlabCap = 128 grains a lane's sum is rounded by at most
+// 128 x 2^-24 of the sum of |weight x impulse|, 27 lanes and the total by twice
+// that of the sum of |impulse| times the |weights|' sum, and the weights' sum
+// differs from 1 by a few 2^-24: 1.7e-5 x 128 x 2^35 = 7.5e7 for grains with
+// an impulse below 2^34 whose weights' sizes add up to less than 2 (they are
+// positive but near the axis and the poles).  Larger ones belong to chunks whose
+// sums are nearly always too large for 32 bits.  A NaN is not calm.
+template <int GEOM>
+__device__ __forceinline__ bool cube_calm(const float D[4], const float w[3][3])
+{
+    constexpr float top = 17179869184.f;
+    bool ok = (fabsf(D[0]) < top) & (fabsf(D[1]) < top) & (fabsf(D[2]) < top) & (fabsf(D[3]) < top);
+    if (GEOM == GEOM_CYL || GEOM == GEOM_SPH) {
+        float s = fabsf(w[0][0]) + fabsf(w[0][1]) + fabsf(w[0][2]);
+        if (GEOM == GEOM_SPH) s *= fabsf(w[1][0]) + fabsf(w[1][1]) + fabsf(w[1][2]);
+        ok = ok & (s < 2.f);
+    }
+    return ok;
+}
+
 // Zone constants of one direction: centre (double and single), inverse width.
 struct __align__(16) CubeZone {
     double c;
@@ -169,8 +194,8 @@ __device__ __forceinline__ void cube_weights(int tsc, bool vol, const float u[3]
 
 // What a grain still needs after the push of its 32: the exact key prediction,
 // or (a grain whose half-step zone is not its key zone, with stale keys) the
-// whole step on its own.
-enum { CUBE_KEY = 1, CUBE_STRAY = 2 };
+// whole step on its own, or the 64-bit rounding of its chunk (cube_calm).
+enum { CUBE_KEY = 1, CUBE_STRAY = 2, CUBE_WILD = 4 };
 
 // The block's constants as the out-of-line paths read them.
 struct CubeRare {
@@ -549,6 +574,7 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
     float moved = 0.f;
     bool big = false, bad = false;
     float2 acc01 = make_float2(0.f, 0.f), acc23 = make_float2(0.f, 0.f);
+    bool wild = false;  // not all of these grains, or of an open chunk before them, are calm
 
     // each warp: a range of the block's zones with an equal share of the work
     // (a zone's roundings cost about as much as 1.5 grains), its grains 32 at
@@ -588,17 +614,18 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
         acc01 = __ffma2_rn(W2, make_float2(De.x, De.y), acc01);
         acc23 = __ffma2_rn(W2, make_float2(De.z, De.w), acc23);
     };
-    // a chunk's sums, rounded, into the box around its host node base
-    auto chunk_end = [&](int base) {
+    // A chunk's sums, rounded, into the box around its host node base.  Sums
+    // below kCubeNarrow take the 32-bit rounding, which gives the same integers
+    // as the 64-bit one at a fraction of its cost; the host's rest has to fit in
+    // 32 bits as well for its modular sum to be exact.  Lane 27 holds the host's
+    // share, which the rest differs from by the rounding of 27 lanes' partial
+    // sums: bounded where the chunk is calm (below), not by the final sums, of
+    // which nothing but that rounding is left where large impulses cancel.
+    auto chunk_end = [&](int base, bool calm) {
         const int lin = base + nlin;
-        // sums below 2^31 (with a margin for their rounding): the 32-bit
-        // rounding gives the same integers as the 64-bit one at a fraction
-        // of its cost.  Lane 27 bounds the host's rest (the host's share of
-        // the impulse plus at most 14 of rounding), so that it, too, fits
-        // in 32 bits and its modular sum is exact.
         const float top = fmaxf(fmaxf(fabsf(acc01.x), fabsf(acc01.y)), fabsf(acc23.x));
-        const bool narrow = top < 2147000000.f && (NCH < 4 || fabsf(acc23.y) < 2147000000.f);
-        if (__all_sync(FULL, narrow) && split) {
+        const bool narrow = top < kCubeNarrow && (NCH < 4 || fabsf(acc23.y) < kCubeNarrow);
+        if (__all_sync(FULL, narrow) && calm) {
             if (lane < 27) {
                 int v[4] = {__float2int_rn(acc01.x), __float2int_rn(acc01.y), __float2int_rn(acc23.x),
                             NCH == 4 ? __float2int_rn(acc23.y) : 0};
@@ -847,16 +874,20 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
                 if (emit) TA.key_out[gi] = nkey;
             }
         }
+        if (!cube_calm<GEOM>(D, w)) todo |= CUBE_WILD;
         if (__any_sync(FULL, todo != 0)) {
             const float value = has_param ? par : A.sp.tau_f[sp];
-            if constexpr (PRED) {
+            wild = wild || __any_sync(FULL, (todo & CUBE_WILD) != 0);
+            todo &= ~CUBE_WILD;
+            if (!__any_sync(FULL, todo != 0)) {
+            } else if constexpr (PRED) {
                 if (todo) big |= cube_rare_predict<GEOM>(TA, R, src, sp, value);
             } else {
                 const CubeRareOut r = cube_rare<GEOM>(TA, R, todo, gi, src, sp, value, nkey,
                                                       reinterpret_cast<float4 *>(rec + lane * kCubeRec));
                 nkey = r.nkey;
-                // strays: one at a time, a chunk of one grain whose weights are
-                // multiplied in the per-grain rule's order
+                // strays: one at a time, a chunk of one grain (no partial sums)
+                // whose weights are multiplied in the per-grain rule's order
                 unsigned strays = __ballot_sync(FULL, r.lin >= 0);
                 if (strays) {
                     __syncwarp();
@@ -868,7 +899,7 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
                         const float W = lane == 13 ? -1.f : fm(e[13 + i % 3], e[4 + i / 3]);
                         acc01 = make_float2(fm(W, e[0]), fm(W, e[1]));
                         acc23 = make_float2(fm(W, e[2]), fm(W, e[3]));
-                        chunk_end(__shfl_sync(FULL, r.lin, k));
+                        chunk_end(__shfl_sync(FULL, r.lin, k), split);
                     }
                     acc01 = s01;
                     acc23 = s23;
@@ -896,6 +927,7 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
         }
         load_grain(gi + 32);
         __syncwarp();
+        const bool quick = split && !wild;
         // ---- deposit: one node per lane, the records in order, a rounding
         // at the end of every chunk
         // groups of four records; stale records after the range's last grain
@@ -917,10 +949,11 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     add(W[j], De[j]);
-                    if (e & (1u << j)) chunk_end(__shfl_sync(FULL, hl, k + j));
+                    if (e & (1u << j)) chunk_end(__shfl_sync(FULL, hl, k + j), quick);
                 }
             }
         }
+        wild = wild && !(ends >> 31);  // only a chunk that these grains left open goes on
         __syncwarp();
     }
     if (big || bad) atomicOr(&A.status[ST_FLAGS], (big ? DUST_FLAG_OVERFLOW : 0) | (bad ? DUST_FLAG_NAN : 0));
