@@ -785,16 +785,16 @@ int run_sort(dust_ctx *ctx, double dt, bool fused)
     // its own: it is bound by memory either way, and the launch no longer counts)
     const int64_t dep_bytes = ctx->ncell * 4 * (int64_t)sizeof(unsigned long long);
     const bool clear_dep = dep_bytes <= kScanClearsDeposit;
+    ctx->keys_ready = false;  // the scan turns the counts into offsets, whatever fails after it
     CU(launch_exclusive_scan(ctx->d_count_next, m, ctx->d_blocksums, ctx->d_cursor, ctx->d_bigseg, ctx->d_count,
                              clear_dep ? ctx->d_dep : nullptr, clear_dep ? dep_bytes : 0, ctx->stream));
-    ctx->count_next_zero = true;
-    ctx->dep_zero = clear_dep;
     CU(launch_sort_scatter<Real>(a, ctx->stream, !fused));
     // fused: the step kernel moves the grains (and then flips the store)
     if (fused) ctx->perm_pending = true;
     else ctx->cur = 1 - ctx->cur;
     std::swap(ctx->d_count, ctx->d_count_next);
-    ctx->keys_ready = false;
+    ctx->count_next_zero = true;
+    ctx->dep_zero = clear_dep;
     return DUST_OK;
 }
 
@@ -2038,11 +2038,12 @@ int capture(dust_batch *b, const double *dt)
     const size_t n = b->ctx.size();
     // host state the capture changes and a failed capture must restore
     struct Saved { int cur; int32_t *count, *count_next; bool keys_ready; double keys_dt;
-                   int64_t launches[dust_ctx::N_GROUPS]; };
+                   bool dep_zero, count_next_zero; int64_t launches[dust_ctx::N_GROUPS]; };
     std::vector<Saved> saved(n);
     for (size_t i = 0; i < n; ++i) {
         dust_ctx *c = b->ctx[i];
-        saved[i] = Saved{c->cur, c->d_count, c->d_count_next, c->keys_ready, c->keys_dt, {}};
+        saved[i] = Saved{c->cur, c->d_count, c->d_count_next, c->keys_ready, c->keys_dt,
+                         c->dep_zero, c->count_next_zero, {}};
         for (int g = 0; g < dust_ctx::N_GROUPS; ++g) saved[i].launches[g] = c->launches[g];
     }
     auto restore = [&](bool state) {
@@ -2057,6 +2058,9 @@ int capture(dust_batch *b, const double *dt)
             c->d_count_next = saved[i].count_next;
             c->keys_ready = saved[i].keys_ready;
             c->keys_dt = saved[i].keys_dt;
+            // the clears were recorded, not run
+            c->dep_zero = saved[i].dep_zero;
+            c->count_next_zero = saved[i].count_next_zero;
         }
     };
     BCU(cudaStreamBeginCapture(b->root, cudaStreamCaptureModeThreadLocal));
