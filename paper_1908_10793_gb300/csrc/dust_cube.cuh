@@ -209,7 +209,10 @@ struct CubeRare {
 
 // First half drift in double precision, boundaries, exact zone search and
 // weights of a grain that is not in its key zone (see slab_exact_first_half).
-// Returns false if it left the grid.
+// The drift and the boundaries are the general path's functions, whose sums have
+// one product each that can be fused; of the volume weights' shell volumes, in
+// double precision, the compiler chooses which.  Returns false if it left the
+// grid.
 template <int GEOM>
 __device__ __forceinline__ bool cube_exact_first_half(const GridDev &g, const PhysDev &ph, double shift, int wk, float h,
                                                       SlabExact &e)

@@ -51,7 +51,8 @@ __device__ __forceinline__ void cube_w_cyl(int tsc, float d, float nu, float w[3
     }
 }
 
-// EXACT: as the path of grains outside their key zone rounds the CIC weights
+// EXACT: the path of grains outside their key zone, which fuses other products of
+// some sums (as the per-grain kernel does)
 template <bool EXACT>
 __device__ __forceinline__ void cube_w_sphr(int tsc, float d, float nu, float w[3])
 {
@@ -60,7 +61,7 @@ __device__ __forceinline__ void cube_w_sphr(int tsc, float d, float nu, float w[
         const float inv = fd(1.f, ff(fm(6.f, s), s, 1.f));
         const float a = fs(0.5f, d), b = fa(0.5f, d);
         const float c0 = ff(fm(4.f, nu), d, ff(d, d, ff(fm(6.f, nu), nu, 2.75f)));
-        const float odd = ff(8.f, nu, fm(3.f, d));
+        const float odd = EXACT ? ff(3.f, d, fm(8.f, nu)) : ff(8.f, nu, fm(3.f, d));
         w[0] = fm(fm(fm(fm(fs(c0, odd), inv), 0.5f), a), a);
         w[2] = fm(fm(fm(fm(fa(c0, odd), inv), 0.5f), b), b);
         const float t = ff(2.f, nu, d);  // the doubling is exact
