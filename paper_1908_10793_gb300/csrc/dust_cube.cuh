@@ -271,6 +271,8 @@ __device__ __noinline__ CubeRareOut cube_rare(const TiledArgs<float> &TA, const 
 #pragma unroll
         for (int d = 0; d < 3; ++d) { ex.q[d] = A.s.q[d][src]; ex.p[d] = A.s.p[d][src]; }
         alive = cube_exact_first_half<GEOM>(g, A.ph, shift_mid_of(A), R.wk, R.h, ex);
+        // removed in its first half drift, in place: its other columns stay
+        const bool stays = !alive && !TA.perm;
 #pragma unroll
         for (int d = 0; d < 3; ++d) { q[d] = ex.q[d]; pnew[d] = ex.p[d]; }
         if (alive) {
@@ -333,8 +335,12 @@ __device__ __noinline__ CubeRareOut cube_rare(const TiledArgs<float> &TA, const 
             atomicAdd(reinterpret_cast<unsigned long long *>(&A.status[ST_REMOVED_LO]), 1ull);
             out.nkey = R.nkeys;
         }
+        if (stays) {
+            O.q[0][gi] = q[0];
+        } else {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) { O.q[d][gi] = q[d]; O.p[d][gi] = pnew[d]; }
+            for (int d = 0; d < 3; ++d) { O.q[d][gi] = q[d]; O.p[d][gi] = pnew[d]; }
+        }
     } else {
 #pragma unroll
         for (int d = 0; d < 3; ++d) { q[d] = O.q[d][gi]; pnew[d] = O.p[d][gi]; }

@@ -1,7 +1,8 @@
 """Grains outside their key zone (keys of the step before, long steps) in the
 spherical geometry: their weights are rounded as the general path rounds them.
 The digests are those of the kernels that pushed such grains by the general
-path's own functions; the inputs use correctly rounded operations only."""
+path's own functions; the inputs use correctly rounded operations only.  And
+grains that leave the grid on that path."""
 import numpy as np
 import pytest
 
@@ -56,3 +57,18 @@ def digests(weight):
 @pytest.mark.parametrize("weight", [I.TSC, I.CIC, I.VOLUME])
 def test_spherical_strays_keep_their_bits(weight):
     assert digests(weight) == GOLDEN[weight]
+
+
+def test_grains_removed_in_place_keep_their_other_columns():
+    """Grains that leave in their first half drift of a step that moves the
+    store in place (the step of length zero before it only sorts)."""
+    w = I.sbox3d("small")
+    w.geom, w.fargo, w.feedback, w.bc = I.CARTESIAN, 0, 0, [I.OUTFLOW] * 3
+    w.species_tau_mode = [I.TAU_CONST]
+    out = w.q[0] > 0.09
+    w.v[0][out] = 10.0
+    w.v[1][out] = 0.125
+    got = run_gpu(w, 2, MIXED, dt=[0.0, 0.01], sort_interval=2)
+    assert out.any() and np.isnan(got["q"][0][out]).all()
+    for d in (1, 2):
+        assert np.array_equal(got["q"][d][out], w.q[d][out])
