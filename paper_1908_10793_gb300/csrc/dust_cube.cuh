@@ -476,6 +476,7 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
     // the block's zones (tile-local keys)
     const int zb0 = (int)(((int64_t)part * tvol) / parts), zb1 = (int)(((int64_t)(part + 1) * tvol) / parts);
     const int64_t kbase = (int64_t)tile * tvol;
+    const int g0 = TA.key_off[kbase + zb0], g1 = TA.key_off[kbase + zb1];  // its grains (fewer than 2^31)
 
     int tc[3];
     tc[0] = tile % g.nt[0];
@@ -496,6 +497,14 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
     float *szhw = reinterpret_cast<float *>(smem_raw + L.hw);
     float *szvl = reinterpret_cast<float *>(smem_raw + L.vl), *szvh = reinterpret_cast<float *>(smem_raw + L.vh);
     unsigned long long *sbar = reinterpret_cast<unsigned long long *>(smem_raw + L.bar);
+    for (int k = threadIdx.x; k < 2 * bvol; k += blockDim.x)
+        reinterpret_cast<uint4 *>(sdep)[k] = make_uint4(0u, 0u, 0u, 0u);
+    // No grains: nothing to stage or deposit.  The test stands after the clear,
+    // which covers the latency of the two offsets (before it: 128^3 box 1.9%
+    // slower); a ring of 200k grains in 192x512x32 zones, most of whose tiles are
+    // empty, takes 151 us a step with the test here and 200 us with one after
+    // the staging.
+    if (g1 <= g0) return;
     // the gas box by one bulk tensor copy, overlapping the tables below
     gas_box_begin<float>(TA.gas_tmap, sgas, o, bvol, sbar, TA.wait_extra_tx);
     const int tsum = T0 + T1 + T2;
@@ -540,8 +549,6 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
     }
     // store positions fit in 32 bits (fewer than 2^31 grains)
     for (int k = zb0 + threadIdx.x; k <= zb1; k += blockDim.x) skoff[k] = TA.key_off[kbase + k];
-    for (int k = threadIdx.x; k < 2 * bvol; k += blockDim.x)
-        reinterpret_cast<uint4 *>(sdep)[k] = make_uint4(0u, 0u, 0u, 0u);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
     float *rec = reinterpret_cast<float *>(smem_raw + L.rec) + warp * (32 * kCubeRec);
@@ -549,7 +556,6 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
     rec[lane * kCubeRec + kCubeOne + 1] = 1.f;
     __syncthreads();
     if (!gas_box_finish<float>(g, A.gas, TA.gas_tmap, sgas, o, B, sbar, A.status, TA.wait_ns)) return;
-    if (skoff[zb1] <= skoff[zb0]) return;  // no grains
 
     CubeBox box;
     box.sdep = sdep;
@@ -557,7 +563,7 @@ __device__ __forceinline__ void cube_tile(const TiledArgs<float> &TA, const int 
     box.bvol = bvol;
     box.B0 = B[0]; box.B1 = B[1];
     box.o0 = o[0]; box.o1 = o[1]; box.o2 = o[2];
-    box.split = skoff[zb1] - skoff[zb0] <= 65535;
+    box.split = g1 - g0 <= 65535;
     CubeRare R;
     R.box = box;
     R.sgas = sgas;
