@@ -116,7 +116,12 @@ __device__ __forceinline__ void cube_w_theta(int tsc, float th, float lo, float 
     w[1] = fs(fs(1.f, w[0]), w[2]);
 }
 
-// Eq. CIC_vol relative to the zone's centre c (see w_vol_f)
+// Eq. CIC_vol relative to the host zone's centre c, for a coordinate x = c + u
+// inside the zone: the shell volume between c and x (written so that it stays
+// accurate for small u) times the inverse shell volume between c and the
+// neighbouring node on that side (ivl, ivh, from vol_shell and vol_node in
+// double precision).  d = 0: the radius (cylindrical R^2, spherical r^3); d = 1:
+// the spherical polar angle.
 template <int GEOM>
 __device__ __forceinline__ void cube_w_vol(int d, float u, float c, float ivl, float ivh, float w[3])
 {

@@ -4,12 +4,12 @@
 // the tile's sort keys (zones), whose grains are contiguous in the store, and
 // walks it in passes of up to kSlabCap grains.
 // Push: one grain per lane over the whole pass (coalesced loads and stores,
-// no per-zone imbalance); the 27-node gather reads the staged gas box (grains
+// no per-zone imbalance); the 9-node gather reads the staged gas box (grains
 // of one zone read the same nodes, so the loads broadcast); each grain leaves
 // a record (weights, deposit impulse) in the warp's shared buffer.  Deposit,
 // ten zones of the pass at a time:
 // three lanes own one zone; lane a keeps, in registers, the accumulators of
-// the nine stencil nodes at x-offset a - 1 and sums the zone's records into
+// the three stencil nodes at x-offset a - 1 and sums the zone's records into
 // them.  A zone's deposit (its run: the grains sorted into it whose half-step
 // host is the zone itself), cut into chunks of kSlabCap grains by rank, is
 // quantised once per chunk and node and added to the shared deposit box; the
@@ -70,9 +70,10 @@ __device__ __forceinline__ void prefetch_grain(const Store &S, int src)
     if (S.species) prefetch_l2(S.species + src);
 }
 
-// A deposit piece too large for the split form of the shared deposit box
-// (below), or from a tile too dense for it: added to the global deposit at
-// the zone of box position lin (x fastest, box of B0 x B1 x ..., origin o).
+// A deposit piece too large for the carry-free counters of the three-
+// dimensional kernels' shared deposit box (dust_cube.cuh): added to the global
+// deposit at the zone of box position lin (x fastest, box of B0 x B1 x ...,
+// origin o).
 static __device__ __noinline__ void box_piece_to_global(const GridDev &g, unsigned long long *dep, int o0, int o1,
                                                  int o2, int B0, int B1, int lin, int ch, long long v)
 {
@@ -284,6 +285,7 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                                           unsigned char *smem_raw, const bool reuse, const int part = 0,
                                           const int parts = 1)
 {
+    static_assert((FLAT == 1 || FLAT == 2) && (GEOM == GEOM_CART || GEOM == GEOM_SB), "two-dimensional boxes only");
     using Sh = SlabShape<FLAT>;
     constexpr int NB = Sh::NB, NC = Sh::NC;
     const StepArgs<float> &A = TA.s;
@@ -297,7 +299,6 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
     // gridded directions, and the weights (the shape copies run TSC)
     auto gd = [&](int d) { return FIX ? (d == 0 || (d == 1 ? FLAT != 1 : FLAT != 2)) : g.n[d] > 1; };
     const int tsc = FIX ? 1 : TA.tsc;
-    const bool vol = FIX ? false : TA.vol != 0;
     // the inline push reads ph; the rare out-of-line paths read the kernel
     // argument (the same values)
     PhysDev ph = A.ph;
@@ -360,48 +361,23 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
     unsigned short *sztab = reinterpret_cast<unsigned short *>(skoff + ((tvol + 32) & ~31));
     float *srec = reinterpret_cast<float *>(sztab + (kSlabThreads / 32) * kSlabCap);  // [warps][13][kRecStride]
     // the tile's zone geometry, per direction d at toff[d]: centre (double and
-    // float) and inverse width; radial centre / width; polar lower edges
+    // float) and inverse width
     const int toff[3] = {0, T0, T0 + T1};
     const int tsum = T0 + T1 + T2;
     double *szcd = reinterpret_cast<double *>(srec + (kSlabThreads / 32) * kRecFields * kRecStride);
     float *szcf = reinterpret_cast<float *>(szcd + tsum);
     float *szif = szcf + tsum;
-    float *sznu = szif + tsum;          // [T0]
-    float *szlo = sznu + T0;        // [T1 + 1]
-    // volume weighting: inverse shell volumes to the lower and upper
-    // neighbouring nodes, radial zones then polar zones ([2 (T0 + T1)])
-    float *szvl = szlo + T1 + 1, *szvh = szvl + T0 + T1;
     unsigned long long *sbar = reinterpret_cast<unsigned long long *>(
-        (reinterpret_cast<uintptr_t>(szvh + T0 + T1) + 7) & ~(uintptr_t)7);
+        (reinterpret_cast<uintptr_t>(szif + tsum) + 7) & ~(uintptr_t)7);
     // the gas box by one bulk tensor copy, overlapping the tables below
     gas_box_begin<float>(TA.gas_tmap, sgas, o, bvol, sbar, TA.wait_extra_tx);
-    for (int t = threadIdx.x; t < tsum + T1 + 1; t += blockDim.x) {
-        if (t < tsum) {
-            const int d = t < toff[1] ? 0 : (t < toff[2] ? 1 : 2);
-            const int z = tc[d] * Td(d) + (t - toff[d]);
-            const bool ok = gd(d) && z < g.n[d];
-            szcd[t] = ok ? g.zc[d][z] : 0.0;
-            szcf[t] = ok ? g.zc_f[d][z] : 0.f;
-            szif[t] = ok ? g.ziw_f[d][z] : 0.f;
-            if (d == 0 && (GEOM == GEOM_CYL || GEOM == GEOM_SPH)) sznu[t] = ok ? g.znu_f[0][z] : 0.f;
-        } else if (GEOM == GEOM_SPH) {
-            const int z = tc[1] * T1 + (t - tsum);
-            szlo[t - tsum] = (g.n[1] > 1 && z <= g.n[1]) ? g.zlo_f[1][z] : 0.f;
-        }
-    }
-    if ((GEOM == GEOM_CYL || GEOM == GEOM_SPH) && vol) {
-        for (int t = threadIdx.x; t < T0 + (GEOM == GEOM_SPH ? T1 : 0); t += blockDim.x) {
-            const int d = t < T0 ? 0 : 1;
-            const int z = d == 0 ? tc[0] * T0 + t : tc[1] * T1 + (t - T0);
-            float vl = 0.f, vh = 0.f;
-            if (z < g.n[d]) {
-                const double c = g.zc[d][z];
-                vl = (float)(1.0 / vol_shell<GEOM>(d, vol_node(g, d, z - 1), c));
-                vh = (float)(1.0 / vol_shell<GEOM>(d, c, vol_node(g, d, z + 1)));
-            }
-            szvl[t] = vl;
-            szvh[t] = vh;
-        }
+    for (int t = threadIdx.x; t < tsum; t += blockDim.x) {
+        const int d = t < toff[1] ? 0 : (t < toff[2] ? 1 : 2);
+        const int z = tc[d] * Td(d) + (t - toff[d]);
+        const bool ok = gd(d) && z < g.n[d];
+        szcd[t] = ok ? g.zc[d][z] : 0.0;
+        szcf[t] = ok ? g.zc_f[d][z] : 0.f;
+        szif[t] = ok ? g.ziw_f[d][z] : 0.f;
     }
     for (int k = threadIdx.x; k < tvol; k += blockDim.x) {
         const int kx = k % T0, ky = (k / T0) % T1, kz = k / (T0 * T1);
@@ -507,29 +483,11 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                 const int lid[3] = {toff[0] + lx, toff[1] + ly, toff[2] + lz};
                 double zcd[3];
                 float zcf[3], zif[3];
-                float znu = 0.f, zlo = 0.f, zhi = 0.f, zhw = 0.f;
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     zcd[d] = szcd[lid[d]];
                     zcf[d] = szcf[lid[d]];
                     zif[d] = szif[lid[d]];
-                }
-                float zvl[2] = {0.f, 0.f}, zvh[2] = {0.f, 0.f};
-                if (GEOM == GEOM_CYL || GEOM == GEOM_SPH) {
-                    znu = sznu[lx];
-                    if (vol) {
-                        zvl[0] = szvl[lx];
-                        zvh[0] = szvh[lx];
-                        if (GEOM == GEOM_SPH) {
-                            zvl[1] = szvl[T0 + ly];
-                            zvh[1] = szvh[T0 + ly];
-                        }
-                    }
-                }
-                if (GEOM == GEOM_SPH) {
-                    zlo = szlo[ly];
-                    zhi = szlo[ly + 1];
-                    zhw = 0.5f / zif[1];
                 }
                 // the grain's weights and deposit impulse for the zone's
                 // owners (zero impulse: the grain deposits by itself)
@@ -565,23 +523,13 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                         if (here) {
 #pragma unroll
                             for (int d = 0; d < 3; ++d) {
-                                if (!gd(d)) continue;
-                                if ((GEOM == GEOM_CYL || GEOM == GEOM_SPH) && d == 0) {
-                                    if (vol) w_vol_f<GEOM>(0, u[0], zcf[0], zvl[0], zvh[0], w[0]);
-                                    else if (GEOM == GEOM_CYL) w_cyl<float>(tsc, dl[0], znu, w[0]);
-                                    else w_sphr<float>(tsc, dl[0], znu, w[0]);
-                                } else if (GEOM == GEOM_SPH && d == 1) {
-                                    if (vol) w_vol_f<GEOM>(1, u[1], zcf[1], zvl[1], zvh[1], w[1]);
-                                    else w_theta<float>(tsc, qf[1], zlo, zhi, u[1], zhw, w[1]);
-                                } else {
-                                    w_cart<float>(tsc, dl[d], w[d]);
-                                }
+                                if (gd(d)) w_cart<float>(tsc, dl[d], w[d]);
                             }
                         } else {
 #pragma unroll
                             for (int d = 0; d < 3; ++d) {
                                 float iwd;
-                                zone_weights<float, GEOM>(g, d, vol ? 2 : (tsc & 1), q[d], host[d], w[d], iwd);
+                                zone_weights<float, GEOM>(g, d, tsc & 1, q[d], host[d], w[d], iwd);
                                 qf[d] = (float)q[d];
                                 int l = host[d] - o[d];
                                 if (gd(d) && g.bc[d] == DUST_BC_PERIODIC) {
@@ -635,20 +583,8 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                             if (gd(d)) { u[d] = __double2float_rn(q[d] - zcd[d]); zc3[d] = zcf[d]; }
                             else { u[d] = 0.f; zc3[d] = (float)q[d]; }
                         }
-                        // first half drift (Eq. exp_midpoint; Eq. drift1_cylindrical;
-                        // spherical r, theta, phi in turn)
-                        if (GEOM == GEOM_CYL) {
-                            inc1[0] = h * pn[0]; u[0] += inc1[0];
-                            const float R = zc3[0] + u[0];
-                            inc1[1] = h * pn[1] / (R * R); u[1] += inc1[1];
-                            inc1[2] = h * pn[2]; u[2] += inc1[2];
-                        } else if (GEOM == GEOM_SPH) {
-                            inc1[0] = h * pn[0]; u[0] += inc1[0];
-                            const float r = zc3[0] + u[0];
-                            inc1[1] = h * pn[1] / (r * r); u[1] += inc1[1];
-                            const float st = sinf(zc3[1] + u[1]);
-                            inc1[2] = h * pn[2] / (r * r * st * st); u[2] += inc1[2];
-                        } else if (GEOM == GEOM_SB) {
+                        // first half drift (Eq. exp_midpoint)
+                        if (GEOM == GEOM_SB) {
                             inc1[0] = h * pn[0]; u[0] += inc1[0];
                             inc1[1] = ph.fargo ? h * (pn[1] - ph.q_om_f * (zc3[0] + u[0])) : h * pn[1];
                             u[1] += inc1[1];
@@ -670,17 +606,7 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
 #pragma unroll
                             for (int d = 0; d < 3; ++d) {
                                 iw[d] = zif[d];
-                                if (!gd(d)) continue;
-                                if ((GEOM == GEOM_CYL || GEOM == GEOM_SPH) && d == 0) {
-                                    if (vol) w_vol_f<GEOM>(0, u[0], zcf[0], zvl[0], zvh[0], w[0]);
-                                    else if (GEOM == GEOM_CYL) w_cyl<float>(tsc, dl[0], znu, w[0]);
-                                    else w_sphr<float>(tsc, dl[0], znu, w[0]);
-                                } else if (GEOM == GEOM_SPH && d == 1) {
-                                    if (vol) w_vol_f<GEOM>(1, u[1], zcf[1], zvl[1], zvh[1], w[1]);
-                                    else w_theta<float>(tsc, qf[1], zlo, zhi, u[1], zhw, w[1]);
-                                } else {
-                                    w_cart<float>(tsc, dl[d], w[d]);
-                                }
+                                if (gd(d)) w_cart<float>(tsc, dl[d], w[d]);
                             }
                         } else {
                             // exact path: double-precision half drift, boundaries
@@ -688,8 +614,7 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                             SlabExact ex;
 #pragma unroll
                             for (int d = 0; d < 3; ++d) { ex.q[d] = q[d]; ex.p[d] = pn[d]; }
-                            const bool in = slab_exact_first_half<GEOM>(g, A.ph, shift_mid_of(A), vol ? 2 : (tsc & 1),
-                                                                        h, ex);
+                            const bool in = slab_exact_first_half<GEOM>(g, A.ph, shift_mid_of(A), tsc & 1, h, ex);
 #pragma unroll
                             for (int d = 0; d < 3; ++d) { q[d] = ex.q[d]; pn[d] = ex.p[d]; inc1[d] = ex.inc[d]; }
                             if (!in) {
@@ -729,7 +654,7 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                             if (gd(d)) inbox &= (l >= 1) && (l <= B[d] - 2);
                         }
                     }
-                    // 27-node gather (Eq. Delta_vp) from the staged gas box; the
+                    // 9-node gather (Eq. Delta_vp) from the staged gas box; the
                     // grains of one zone read the same nodes (broadcast loads)
                     if (inbox) {
                         // channels in pairs on the packed single-precision
@@ -790,18 +715,9 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                     float pp[3], acc3[3], dH[3], inc2[3];
                     kick_any<float, GEOM>(ph, qf, pn, vg, tau, dt, E, cg, h1, pp, acc3, dH);
                     if (ingroup) {
-                        // second half drift with the half-step metric factors, then
+                        // second half drift with the half-step coordinates, then
                         // one double-precision update by the summed increment
-                        if (GEOM == GEOM_CYL) {
-                            inc2[0] = h * pp[0];
-                            inc2[1] = h * pp[1] / (qf[0] * qf[0]);
-                            inc2[2] = h * pp[2];
-                        } else if (GEOM == GEOM_SPH) {
-                            const float st = sinf(qf[1]);
-                            inc2[0] = h * pp[0];
-                            inc2[1] = h * pp[1] / (qf[0] * qf[0]);
-                            inc2[2] = h * pp[2] / (qf[0] * qf[0] * st * st);
-                        } else if (GEOM == GEOM_SB) {
+                        if (GEOM == GEOM_SB) {
                             inc2[0] = h * pp[0];
                             inc2[1] = ph.fargo ? h * (pp[1] - ph.q_om_f * qf[0]) : h * pp[1];
                             inc2[2] = h * pp[2];
@@ -894,18 +810,7 @@ __device__ __forceinline__ bool slab_tile(const TiledArgs<float> &TA, const int 
                             float un[3];
 #pragma unroll
                             for (int d = 0; d < 3; ++d) un[d] = u[d] + inc2[d];
-                            if (GEOM == GEOM_CYL) {
-                                un[0] += h * pnew[0];
-                                const float R = zc3[0] + un[0];
-                                un[1] += h * pnew[1] / (R * R);
-                                un[2] += h * pnew[2];
-                            } else if (GEOM == GEOM_SPH) {
-                                un[0] += h * pnew[0];
-                                const float r = zc3[0] + un[0];
-                                un[1] += h * pnew[1] / (r * r);
-                                const float st = sinf(zc3[1] + un[1]);
-                                un[2] += h * pnew[2] / (r * r * st * st);
-                            } else if (GEOM == GEOM_SB) {
+                            if (GEOM == GEOM_SB) {
                                 un[0] += h * pnew[0];
                                 un[1] += ph.fargo ? h * (pnew[1] - ph.q_om_f * (zc3[0] + un[0])) : h * pnew[1];
                                 un[2] += h * pnew[2];
@@ -1176,12 +1081,12 @@ step_slab_kernel(const __grid_constant__ TiledArgs<float> TA, const int parts)
 // Gas predictor on the slab layout (Sec. 3.1): one tile per block, the
 // chunk rule for grains whose x^n lies in their key zone, the per-grain rule
 // for the others.
-template <int GEOM, int FLAT, int TX = 0, int TY = 0, int TZ = 0>
+template <int GEOM, int FLAT>
 __global__ void __launch_bounds__(kSlabThreads, 2)
 predict_slab_kernel(const __grid_constant__ TiledArgs<float> TA, const int parts)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    slab_tile<GEOM, FLAT, 1, TX, TY, TZ, true>(TA, blockIdx.x / parts, gridDim.x / parts, smem_raw, false,
+    slab_tile<GEOM, FLAT, 1, 0, 0, 0, true>(TA, blockIdx.x / parts, gridDim.x / parts, smem_raw, false,
                                                blockIdx.x % parts, parts);
 }
 
@@ -1207,8 +1112,7 @@ inline size_t slab_smem_bytes(const GridDev &g)
            (size_t)((g.tvol + 31) & ~31) * sizeof(int) + (size_t)((g.tvol + 32) & ~31) * sizeof(int) +
            (size_t)(kSlabThreads / 32) * kSlabCap * sizeof(unsigned short) +
            (size_t)(kSlabThreads / 32) * kRecFields * kRecStride * sizeof(float) +
-           tsum * (sizeof(double) + 2 * sizeof(float)) + ((size_t)g.T[0] + g.T[1] + 1) * sizeof(float) +
-           2 * ((size_t)g.T[0] + g.T[1]) * sizeof(float) +
+           tsum * (sizeof(double) + 2 * sizeof(float)) +
            16;  // the bulk copy's transaction barrier (8-byte aligned)
 }
 
