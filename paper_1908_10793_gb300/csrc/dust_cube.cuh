@@ -22,8 +22,8 @@
 // nodes each held 36), all lanes are in the same zone at the same time, so
 // uneven zones cost nothing, and the push runs on 32 lanes whatever the zones
 // hold.  Step kernel, before (three owner lanes per zone) and with this one:
-// 128^3 box 1434 -> 1191 us, 50M-grain cylindrical disk (two grains per zone)
-// 6943 -> 5944 us, 33M-grain spherical disk 6214 -> 4601 us, 50x37x29 box 120 ->
+// 128^3 box 1434 -> 1183 us, 50M-grain cylindrical disk (two grains per zone)
+// 6943 -> 5940 us, 33M-grain spherical disk 6214 -> 4597 us, 50x37x29 box 120 ->
 // 70 us, one zone in two hundred grains deep (200k grains) 2761 -> 240 us.
 // Three blocks per SM (80 registers) spill: 1635 us; 320 or 384 threads: 1430
 // and 1580 us.
