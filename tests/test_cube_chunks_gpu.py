@@ -1,11 +1,13 @@
 """The three-dimensional slab kernels' chunk sums: the 32-bit rounding path is
 taken only where the host zone's rest cannot leave 32 bits, so its integers are
-those of the 64-bit path."""
+those of the 64-bit path; and the carry-free deposit box gives those of the box
+of int64 words."""
 import numpy as np
 import pytest
 
 from paper_1908_10793_gb300 import inputs as I
 from parity_util import run_gpu
+from test_cube_gpu import _box
 from test_parity_gpu import MIXED
 
 pytestmark = pytest.mark.gpu
@@ -59,3 +61,17 @@ def test_predictor_chunks_of_cancelling_impulses(tile):
                      for d in (False, True))
     for a, b in zip(sparse["v"], dense["v"]):
         assert np.array_equal(a, b[:len(a)])
+
+
+@pytest.mark.parametrize("predictor", [0, 1])
+def test_deposit_boxes_agree(predictor):
+    """About 1170 grains in each of 8^3 zones: one tile's eight parts hold more
+    than 65535 grains each (int64 words), the parts of smaller tiles fewer
+    (carry-free counters)."""
+    w = _box((8, 8, 8), 600001)
+    words = run_gpu(w, 2, MIXED, gas_predictor=predictor)
+    counters = run_gpu(w, 2, MIXED, gas_predictor=predictor, tile=(4, 3, 5))
+    assert np.array_equal(words["fixed"], counters["fixed"])
+    for k in ("q", "v"):
+        for a, b in zip(words[k], counters[k]):
+            assert np.array_equal(a, b)
